@@ -53,6 +53,44 @@ struct Vec<float, 4> {
     }
 };
 
+// (double)x without the FP64 pipe, on which a conversion costs as much as an
+// addition (two per SM cycle on GB300): a normal binary32 number's bits are
+// its binary64 number's, the exponent rebiased.
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// (float)x, rounded to nearest even, likewise on the integer units: the
+// value's low 29 bits decide. Outside the range of normal binary32 numbers
+// the conversion instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned m = h & 0x7fffffffu;
+    if (m < 0x38100000u || m >= 0x47e00000u) return __double2float_rn(x);
+    unsigned r = ((m - 0x38000000u) << 3) | (l >> 29);
+    const unsigned rest = l << 3;
+    r += (rest > 0x80000000u || (rest == 0x80000000u && (r & 1u))) ? 1u : 0u;
+    return __uint_as_float((h & 0x80000000u) | r);
+}
+__device__ __forceinline__ void narrow_to(float& d, double x) { d = narrow(x); }
+__device__ __forceinline__ void narrow_to(double& d, double x) { d = x; }
+
+// Density and velocity of one member's f (g = f - w with SHIFT), FP64: 16
+// additions, one division and two products.
+template <bool SHIFT>
+__device__ __forceinline__ void moments_of(const double (&g)[9], double& r, double& ux, double& uy) {
+    const double d56 = g[5] - g[6], d78 = g[7] - g[8];
+    const double jx = (g[1] - g[2]) + (d56 + d78), jy = (g[3] - g[4]) + (d56 - d78);
+    r = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    if (SHIFT) r += 1.0;
+    const double ir = 1.0 / r;
+    ux = jx * ir;
+    uy = jy * ir;
+}
+
 // Work item t of a lattice kernel -> member group mv (of kv per cell), cell,
 // and its coordinates (x, y). The divisions run in 32 bits while t fits
 // (64-bit integer division is emulated and costs several times more).
