@@ -104,8 +104,9 @@ cudaError_t launch_mean_velocity(const void* f, int fp32, int nx, int ny, int k,
 cudaError_t launch_set_equilibrium(void* f, int fp32, int nx, int ny, int k,
                                    const double* rho, const double* u, const double* v,
                                    cudaStream_t s);
-cudaError_t launch_store_f(void* f, int fp32, const double* src, size_t n, cudaStream_t s);
-cudaError_t launch_load_f(const void* f, int fp32, double* dst, size_t n, cudaStream_t s);
+// FP64 f [9][ny][nx][k] (n values) to the binary32 state and back.
+cudaError_t launch_store_f(void* f, const double* src, size_t n, cudaStream_t s);
+cudaError_t launch_load_f(const void* f, double* dst, size_t n, cudaStream_t s);
 cudaError_t launch_store_force(void* dst, int fp32, const double* src, size_t n,
                                cudaStream_t s);
 

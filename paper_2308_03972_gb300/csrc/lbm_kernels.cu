@@ -286,6 +286,9 @@ cudaError_t launch_step_v(const T* fin, T* fout, const T* force, const LbmParams
 }
 
 // Moments from the stored state: rho = sum f, u = sum f c / rho, in FP64.
+// Bound by the FP64 pipe (two operations per SM cycle), so the nine
+// conversions run on the integer units and the sums share their differences:
+// 436 -> 291 us at 256^2 x 64 in binary32.
 template <typename T, bool SHIFT>
 __global__ void moments_kernel(const T* __restrict__ f, int nx, int ny, int k,
                                double* __restrict__ rho, double* __restrict__ u,
@@ -293,31 +296,22 @@ __global__ void moments_kernel(const T* __restrict__ f, int nx, int ny, int k,
     const size_t n = (size_t)nx * ny * k;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double g[9];
+    double g[9], r, ux, uy;
 #pragma unroll
-    for (int a = 0; a < 9; ++a) g[a] = (double)f[a * n + i];
-    double r = 0.0, jx = 0.0, jy = 0.0;
-#pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        r += g[a];
-        jx += d2q9_cx(a) * g[a];
-        jy += d2q9_cy(a) * g[a];
-    }
-    if (SHIFT) r += 1.0;
-    const double ux = jx / r, uy = jy / r;
+    for (int a = 0; a < 9; ++a) g[a] = widen(f[a * n + i]);
+    moments_of<SHIFT>(g, r, ux, uy);
     if (rho) rho[i] = r;
     if (u) u[i] = ux;
     if (v) v[i] = uy;
     if (!(ux * ux + uy * uy <= kUMax2) || !(r > 0.0)) atomicOr(flags, FLAG_DIVERGED);
 }
 
-// Ensemble-mean velocity: one warp per cell, lanes over members. A member's
-// moments are taken in the precision of the stored state (FP64 here; the
-// binary32 shifted state g = f - w has its own kernel below, whose moments
-// match that state's storage error, ~1e-9 absolute in u); the member mean
-// is summed in FP64.
-template <typename T, bool SHIFT>
-__global__ void mean_velocity_kernel(const T* __restrict__ f, int nx, int ny, int k,
+// Ensemble-mean velocity of an FP64 state: one warp per cell, lanes over
+// members, moments and sum in FP64. The binary32 shifted state g = f - w has
+// its own kernel below, whose moments match that state's storage error
+// (~1e-9 absolute in u). One division per member: 479 -> 336 us at
+// 256^2 x 64.
+__global__ void mean_velocity_kernel(const double* __restrict__ f, int nx, int ny, int k,
                                      double* __restrict__ um, double* __restrict__ vm,
                                      int* __restrict__ flags) {
     const long long cell = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -328,21 +322,13 @@ __global__ void mean_velocity_kernel(const T* __restrict__ f, int nx, int ny, in
     bool bad = false;
     for (int m = lane; m < k; m += 32) {
         const size_t i = (size_t)cell * k + m;
-        T r = T(0), jx = T(0), jy = T(0);
+        double g[9], r, ux, uy;
 #pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const T g = f[a * n + i];
-            r += g;
-            jx += T(d2q9_cx(a)) * g;
-            jy += T(d2q9_cy(a)) * g;
-        }
-        if (SHIFT) r += T(1);
-        const T ux = jx / r, uy = jy / r;
-        su += (double)ux;
-        sv += (double)uy;
-        // The divergence test in the state's precision, as the LBM step
-        // makes it (0.25 is exact in binary32).
-        bad |= !(ux * ux + uy * uy <= T(kUMax2)) || !(r > T(0));
+        for (int a = 0; a < 9; ++a) g[a] = f[a * n + i];
+        moments_of<false>(g, r, ux, uy);
+        su += ux;
+        sv += uy;
+        bad |= !(ux * ux + uy * uy <= kUMax2) || !(r > 0.0);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -432,41 +418,65 @@ __global__ void mean_velocity_f32_kernel(const float* __restrict__ f, int nx, in
     }
 }
 
+// f^eq(rho, u, v) of every member: f^eq_a - w_a = w_a (A + rho (4.5 (c.u)^2 +
+// 3 c.u)), A = rho - 1 - 1.5 rho u.u, in FP64. Opposite directions share their
+// even part; on a diagonal 4.5 (ux +- uy)^2 = 4.5 u.u +- 9 ux uy. Bound by
+// the FP64 pipe: about 30 operations per member-cell (and 9 additions of w in
+// FP64 storage), the conversions to binary32 on the integer units:
+// 517 -> 295 us at 256^2 x 64 in FP64.
 template <typename T, bool SHIFT>
 __global__ void equilibrium_kernel(T* __restrict__ f, size_t n, const double* __restrict__ rho,
                                    const double* __restrict__ u, const double* __restrict__ v) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double r = rho ? rho[i] : 1.0;
     const double ux = u ? u[i] : 0.0, uy = v ? v[i] : 0.0;
-    const double uu = ux * ux + uy * uy;
-#pragma unroll
-    for (int a = 0; a < 9; ++a) {
-        const double cu = d2q9_cx(a) * ux + d2q9_cy(a) * uy;
-        const double w = d2q9_w(a);
-        // f^eq - w = w ((rho - 1) + rho (3 cu + 9/2 cu^2 - 3/2 uu)).
-        const double dev = w * ((r - 1.0) + r * (3.0 * cu + 4.5 * cu * cu - 1.5 * uu));
-        f[a * n + i] = SHIFT ? (T)dev : (T)(w + dev);
+    double xx = ux * ux, yy = uy * uy, xy = ux * uy, lx = ux, ly = uy, r1 = 0.0;
+    if (rho) {
+        const double r = rho[i];
+        r1 = r - 1.0;
+        xx *= r;
+        yy *= r;
+        xy *= r;
+        lx *= r;
+        ly *= r;
     }
+    const double uu = xx + yy;
+    const double A = fma(-1.5, uu, r1);
+    double d[9];
+    d[0] = (4.0 / 9.0) * A;
+    const double a1 = (1.0 / 9.0) * A;
+    const double ex = fma(0.5, xx, a1), ey = fma(0.5, yy, a1);
+    d[1] = fma(1.0 / 3.0, lx, ex);
+    d[2] = fma(-1.0 / 3.0, lx, ex);
+    d[3] = fma(1.0 / 3.0, ly, ey);
+    d[4] = fma(-1.0 / 3.0, ly, ey);
+    const double dg = (1.0 / 36.0) * fma(4.5, uu, A);
+    const double e5 = fma(0.25, xy, dg), e7 = fma(-0.25, xy, dg);
+    const double lp = lx + ly, lm = lx - ly;
+    d[5] = fma(1.0 / 12.0, lp, e5);
+    d[6] = fma(-1.0 / 12.0, lp, e5);
+    d[7] = fma(1.0 / 12.0, lm, e7);
+    d[8] = fma(-1.0 / 12.0, lm, e7);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) narrow_to(f[a * n + i], SHIFT ? d[a] : d2q9_w(a) + d[a]);
 }
 
-// FP64 f [9][ny][nx][k] <-> stored representation (plane = ny nx k).
-template <typename T, bool SHIFT>
-__global__ void store_f_kernel(T* __restrict__ dst, const double* __restrict__ src, size_t n,
-                               size_t plane) {
+// FP64 f [9][ny][nx][k] <-> g = f - w in binary32 (plane = ny nx k; grid y = 9).
+// One FP64 addition per value is left on the FP64 pipe; the conversions run on
+// the integer units. With the equilibrium above, setting a
+// 256^2 x 64 binary32 ensemble and reading it back went from 744 to 393 us.
+__global__ void store_f_kernel(float* __restrict__ dst, const double* __restrict__ src, size_t plane) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int a = (int)(i / plane);
-    dst[i] = SHIFT ? (T)(src[i] - d2q9_w(a)) : (T)src[i];
+    if (i >= plane) return;
+    const size_t at = blockIdx.y * plane + i;
+    dst[at] = narrow(src[at] - d2q9_w(blockIdx.y));
 }
 
-template <typename T, bool SHIFT>
-__global__ void load_f_kernel(double* __restrict__ dst, const T* __restrict__ src, size_t n,
-                              size_t plane) {
+__global__ void load_f_kernel(double* __restrict__ dst, const float* __restrict__ src, size_t plane) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int a = (int)(i / plane);
-    dst[i] = SHIFT ? (double)src[i] + d2q9_w(a) : (double)src[i];
+    if (i >= plane) return;
+    const size_t at = blockIdx.y * plane + i;
+    dst[at] = widen(src[at]) + d2q9_w(blockIdx.y);
 }
 
 __global__ void store_force_f32(float* __restrict__ dst, const double* __restrict__ src, size_t n) {
@@ -561,7 +571,7 @@ cudaError_t launch_mean_velocity(const void* f, int fp32, int nx, int ny, int k,
         mean_velocity_f32_kernel<<<blocks_for(threads, 256), 256, 0, s>>>((const float*)f, nx, ny, k, u, v,
                                                                           flags);
     else
-        mean_velocity_kernel<double, false><<<blocks_for(threads, 256), 256, 0, s>>>(
+        mean_velocity_kernel<<<blocks_for(threads, 256), 256, 0, s>>>(
             (const double*)f, nx, ny, k, u, v, flags);
     return cudaGetLastError();
 }
@@ -578,24 +588,15 @@ cudaError_t launch_set_equilibrium(void* f, int fp32, int nx, int ny, int k, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_store_f(void* f, int fp32, const double* src, size_t n, cudaStream_t s) {
-    const size_t plane = n / 9;
+cudaError_t launch_store_f(void* f, const double* src, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    if (fp32)
-        store_f_kernel<float, true><<<blocks_for(n, 256), 256, 0, s>>>((float*)f, src, n, plane);
-    else
-        store_f_kernel<double, false><<<blocks_for(n, 256), 256, 0, s>>>((double*)f, src, n, plane);
+    store_f_kernel<<<dim3(blocks_for(n / 9, 256), 9), 256, 0, s>>>((float*)f, src, n / 9);
     return cudaGetLastError();
 }
 
-cudaError_t launch_load_f(const void* f, int fp32, double* dst, size_t n, cudaStream_t s) {
-    const size_t plane = n / 9;
+cudaError_t launch_load_f(const void* f, double* dst, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    if (fp32)
-        load_f_kernel<float, true><<<blocks_for(n, 256), 256, 0, s>>>(dst, (const float*)f, n, plane);
-    else
-        load_f_kernel<double, false><<<blocks_for(n, 256), 256, 0, s>>>(dst, (const double*)f, n,
-                                                                       plane);
+    load_f_kernel<<<dim3(blocks_for(n / 9, 256), 9), 256, 0, s>>>(dst, (const float*)f, n / 9);
     return cudaGetLastError();
 }
 

@@ -1006,11 +1006,11 @@ int lbm_get_f(lbm_ctx* c, double* f, int ptr_kind) {
                               c->stream),
            "copying state out");
     } else if (ptr_kind == LBM_PTR_DEVICE) {
-        CK(c, launch_load_f(c->f[c->cur], 1, f, n, c->stream), "converting state");
+        CK(c, launch_load_f(c->f[c->cur], f, n, c->stream), "converting state");
     } else {
         int st = ensure_stage(c);
         if (st) return st;
-        CK(c, launch_load_f(c->f[c->cur], 1, c->stage, n, c->stream), "converting state");
+        CK(c, launch_load_f(c->f[c->cur], c->stage, n, c->stream), "converting state");
         CK(c, cudaMemcpyAsync(f, c->stage, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream),
            "copying state out");
     }
@@ -1037,7 +1037,7 @@ int lbm_set_f(lbm_ctx* c, const double* f, int ptr_kind) {
             if ((st = copy_in(c, c->stage, f, n, ptr_kind))) return st;
             src = c->stage;
         }
-        CK(c, launch_store_f(c->f[c->cur], 1, src, n, c->stream), "converting state");
+        CK(c, launch_store_f(c->f[c->cur], src, n, c->stream), "converting state");
     }
     if (ptr_kind == LBM_PTR_HOST) CK(c, cudaStreamSynchronize(c->stream), "synchronising");
     c->observed = false;
