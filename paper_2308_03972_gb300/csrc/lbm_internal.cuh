@@ -166,11 +166,11 @@ cudaError_t launch_analyze_runs_fp64(double* f, int nx, int ny, int k, const Obs
                                      const AnalyzeAux* aux, int pipe_runs, cudaStream_t s);
 // FP64 warm-started analysis of the nruns * run_len grid points of the runs
 // run0.. (chunk-local basis Yg [.][ns][ns], eigenvalue estimates lamg
-// [.][ns] with -1 marking a point with no observation in range, union
-// lists rinfo [.][info_stride]).
-cudaError_t launch_run_fp64(double* f, int nx, int ny, int k, const ObsParams& o, double d_cut, double beta,
+// [.][ns] with -1 marking a point with no observation in range, weights wg
+// [.][ns], union lists rinfo [.][info_stride]).
+cudaError_t launch_run_fp64(double* f, int nx, int ny, int k, const ObsParams& o, double beta,
                             int run_len, int run0, int nruns, int ns, const float* Yg, const float* lamg,
-                            const int* rinfo, int info_stride, int* flags, cudaStream_t s);
+                            const double* wg, const int* rinfo, int info_stride, int* flags, cudaStream_t s);
 // The run analyses of several experiments (one lattice, state and
 // observation set each) in batched launches: kernel J over the runs of
 // every experiment of a size class in one launch, then kernel F over their

@@ -30,6 +30,7 @@
 #include "lbm_internal.cuh"
 #include "letkf_device.cuh"
 #include "tc_ptx.cuh"
+#include "vec.cuh"
 
 namespace lbmgpu {
 namespace {
@@ -186,12 +187,12 @@ __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 // warp. Only what symmetry requires is updated: each rotated pair's 2 x 2
 // diagonal block analytically (a_pp - t a_pq, a_qq + t a_pq, 0), the
 // off-diagonal 2 x 2 blocks (P, Q), P < Q, as J_P^T X J_Q (mirrored), and the
-// rows of U. A rotation is skipped when |a_pq| <= rel ||A||_F; the solve ends
-// after a sweep without one. n <= 64 (at most 32 pairs). Returns the number
+// rows of U. A rotation is skipped when |a_pq| <= max(rel ||A||_F, least);
+// the solve ends after a sweep without one. n <= 64 (at most 32 pairs). Returns the number
 // of sweeps (the last one rotating nothing), or -1 if max_sweeps was reached.
 template <typename R>
 __device__ int jacobi_sym_warp(R* A, R* U, int n, int ld, int lane, R* rc, R* rs, int* rp,
-                                int* rq, R rel, int max_sweeps) {
+                                int* rq, R rel, R least, int max_sweeps) {
     const int np = n + (n & 1);
     const int half = np / 2;
     const int nb = half * (half - 1) / 2;
@@ -199,7 +200,8 @@ __device__ int jacobi_sym_warp(R* A, R* U, int n, int ld, int lane, R* rc, R* rs
     for (int c = lane; c < n; c += 32)
         for (int i = 0; i < n; ++i) fro += A[i * ld + c] * A[i * ld + c];
     fro = warp_sum(fro);
-    const R thresh = rel * sqrt(fro);
+    const R rule = rel * sqrt(fro);
+    const R thresh = rule > least ? rule : least;
     for (int sweep = 0; sweep < max_sweeps; ++sweep) {
         bool any_sweep = false;
         for (int r = 0; r + 1 < np; ++r) {
@@ -453,6 +455,7 @@ struct AnaSmem {
     double* zv;    // [16]
     double* rc;    // [NM / 2]
     double* rs;    // [NM / 2]
+    float* Zf;     // [9][NM] binary32
     int* rp;       // [NM / 2]
     int* rq;       // [NM / 2]
     int* lidx;     // [nl]
@@ -460,7 +463,7 @@ struct AnaSmem {
     __host__ __device__ static size_t bytes(int k, int nl) {
         const size_t d = 2 * (size_t)NM * kLd + 9 * (size_t)k + 16 + 2 * (size_t)nl + 5 * NM +
                          18 * (size_t)NM + 16 + NM;
-        return d * sizeof(double) + (size_t)(NM + nl) * sizeof(int);
+        return d * sizeof(double) + 9 * NM * sizeof(float) + (size_t)(NM + nl) * sizeof(int);
     }
     __device__ void carve(unsigned char* raw, int k, int nl) {
         double* p = reinterpret_cast<double*>(raw);
@@ -496,7 +499,8 @@ struct AnaSmem {
         p += NM / 2;
         rs = p;
         p += NM / 2;
-        int* ip = reinterpret_cast<int*>(p);
+        Zf = reinterpret_cast<float*>(p);
+        int* ip = reinterpret_cast<int*>(Zf + 9 * NM);
         rp = ip;
         ip += NM / 2;
         rq = ip;
@@ -505,47 +509,97 @@ struct AnaSmem {
     }
 };
 
+// 1 / d from the binary32 reciprocal and one Newton step (relative error
+// ~1e-13; here it scales entries that are ~1e-6 of the result).
+__device__ __forceinline__ double recip_step(double d) {
+    if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
+    const double r = widen(__fdividef(1.0f, narrow(d)));
+    return fma(r, fma(-d, r, 1.0), r);
+}
+
+// Largest off-diagonal entry (relative to a = (k-1)/beta) that the FP64
+// transform below takes as it is.
+constexpr double kOffDiag = 1e-6;
+
 // Observation-space transform and update of one grid point (FP64), after
-// the eigensolve: A holds S = U^T A U (nearly diagonal), U the basis;
-// lidx, lsq, ldh the n local scalars (zero weight on padding), dX and
-// xbar the staged state; the result goes to fc. One warp.
+// the eigensolve: A holds S = U^T A U = diag(s) + O, U the basis; lidx, lsq,
+// ldh the n local scalars (zero weight on padding), dX and xbar the staged
+// state; the result goes to fc. One warp.
+//
+// The matrix functions are taken to second order in O. With X = (aI + S)^{1/2},
+// u_i = sqrt(a + s_i), r = sqrt(a):
+//   h(S) = (aI + S)^{-1}, applied to a vector: h0 (t - O h0 t + O h0 O h0 t);
+//   g(S) = ((aI+S)^{-1/2} - a^{-1/2} I) S^{-1} = -(1/r) (X^2 + r X)^{-1}
+//        = -(1/r) (K0 + P)^{-1}, K0 = diag(1/alpha), alpha_i = 1/(u_i (u_i + r)),
+//   P = O + r (X1 + X2), X1_ij = O_ij / (u_i + u_j), X2_ij = -(X1^2)_ij / (u_i + u_j)
+// (X^2 = aI + S to second order), and (K0 + P)^{-1} = alpha - alpha P alpha +
+// alpha P alpha P alpha. What is neglected is third order: with |O_ij| <=
+// 1e-6 a (the eigensolve's stopping rule, or 3e-8 ||A||_F where that is
+// more) below 1e-14 of the transform, where the first-order functions that
+// stood here left 3e-13 at 3e-8 ||A||_F. So the eigensolve may stop an order
+// and a half earlier: from kernel J's basis it usually has nothing left to
+// rotate. Second-order terms (< 1e-9 of the result) run in binary32, scaled
+// by a so that they stay in its range. Once X1 is formed only the upper
+// triangle of A is used (P, FP64); each entry below the diagonal holds the
+// binary32 factor (X1 / r, then P / a) of the mirrored one.
 template <int NM>
 __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t plane, int k, int n,
                                 double aa, double beta, const ObsParams& o, int lane) {
     constexpr int ld = AnaSmem<NM>::kLd;
     double* A = sm.A;
     double* U = sm.U;
-    // With u_i = sqrt(a + s_ii), h(s) = 1/(a+s) and g(s) = ((a+s)^{-1/2} - a^{-1/2}) / s:
-    //   h(S)_ii = 1/u_i^2, h(S)_ij = -s_ij / (u_i^2 u_j^2),
-    //   g(S)_ii = -alpha_i / r, g(S)_ij = s_ij (u_i+u_j+r) alpha_i alpha_j / (r (u_i+u_j)),
-    // alpha_i = 1 / (u_i (u_i + r)), r = sqrt(a).
+    auto up = [&](int i, int j) -> double& { return A[i < j ? i * ld + j : j * ld + i]; };
+    auto low = [&](int i, int j) -> float& { return *reinterpret_cast<float*>(A + (i > j ? i * ld + j : j * ld + i)); };
     const double rr = sqrt(aa);
     const double ir = 1.0 / rr;
     for (int c = lane; c < n; c += 32) {
         const double sii = A[c * ld + c];
         const double u = sqrt(aa + sii);
         sm.v3[c] = u;
-        sm.v4[c] = 1.0 / (aa + sii);      // h_i
+        const double hi = 1.0 / (aa + sii);
+        sm.v4[c] = hi;
         sm.v5[c] = 1.0 / (u * (u + rr));  // alpha_i
         double t = 0.0;
         for (int l = 0; l < n; ++l) t += U[l * ld + c] * sm.ldh[l];
-        sm.v1[c] = t;  // t1 = U^T d-hat
+        sm.v1[c] = hi * t;  // h0 t1, t1 = U^T d-hat
     }
     __syncwarp();
     for (int c = lane; c < n; c += 32) {
         double t = 0.0;
         for (int j = 0; j < n; ++j)
-            if (j != c) t += A[c * ld + j] * (sm.v4[j] * sm.v1[j]);
-        sm.v2[c] = sm.v4[c] * (sm.v1[c] - t);  // t2 = h(S) t1
+            if (j != c) t += A[c * ld + j] * sm.v1[j];
+        sm.v2[c] = sm.v4[c] * t;  // w1 = h0 O h0 t1
     }
     __syncwarp();
+    {
+        // t2 = h(S) t1 = h0 t1 - w1 + h0 O w1
+        double t2[(NM + 31) / 32];
+#pragma unroll
+        for (int q = 0; q < (NM + 31) / 32; ++q) {
+            const int c = lane + 32 * q;
+            if (c >= n) break;
+            double t = 0.0;
+            for (int j = 0; j < n; ++j)
+                if (j != c) t += A[c * ld + j] * sm.v2[j];
+            t2[q] = fma(sm.v4[c], t, sm.v1[c] - sm.v2[c]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < (NM + 31) / 32; ++q)
+            if (lane + 32 * q < n) sm.v2[lane + 32 * q] = t2[q];
+    }
+    __syncwarp();
+    // X1 and the first-order part of P over O.
     for (int c = lane; c < n; c += 32) {
-        // g(S), column c, over S (each column is read and written by one lane).
-        const double ui = sm.v3[c];
-        const double ai = sm.v5[c];
-        for (int j = 0; j < n; ++j) {
-            const double uj = sm.v3[j];
-            A[j * ld + c] = (j == c) ? -ai * ir : A[j * ld + c] * (ui + uj + rr) * ai * sm.v5[j] * ir / (ui + uj);
+        const double uc = sm.v3[c];
+        // Pairs {c, c + d mod n}, d <= n / 2: each lane has the same number.
+        for (int d = 1; 2 * d <= n; ++d) {
+            if (2 * d == n && c >= d) break;
+            const int j = c + d < n ? c + d : c + d - n;
+            const double off = A[j * ld + c];
+            const double x1 = off * recip_step(uc + sm.v3[j]);
+            up(j, c) = fma(rr, x1, off);
+            low(j, c) = narrow(x1 * ir);
         }
         double t = 0.0;
         for (int l = 0; l < n; ++l) t += U[c * ld + l] * sm.v2[l];
@@ -564,35 +618,96 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
         for (int a = 0; a < 9; ++a) sm.Z[a * NM + c] = sm.lsq[c] * acc[a];
     }
     __syncwarp();
-    // zv = Z v (= dX w-bar); B = Z U.
+    // P += r X2 = -a q / (u_i / r + u_j / r), q = (X1 / r)^2 (its diagonal,
+    // too: P's diagonal is that term alone).
+    for (int c = lane; c < n; c += 32) {
+        const float uc = narrow(sm.v3[c] * ir);
+        for (int d = 0; 2 * d <= n; ++d) {
+            if (2 * d == n && c >= d) break;
+            const int j = c + d < n ? c + d : c + d - n;
+            float q0 = 0.0f, q1 = 0.0f;
+            for (int l = 0; l < n; ++l) {
+                if (l == c || l == j) continue;
+                const float xa = low(l, c), xb = low(l, j);
+                if (l & 1)
+                    q1 = fmaf(xa, xb, q1);
+                else
+                    q0 = fmaf(xa, xb, q0);
+            }
+            const float x2 = __fdividef(q0 + q1, uc + narrow(sm.v3[j] * ir));
+            const double p1 = d == 0 ? 0.0 : up(j, c);
+            up(j, c) = fma(-aa, widen(x2), p1);
+        }
+    }
+    __syncwarp();
+    // P / a in binary32 below the diagonal; zv = Z v (= dX w-bar);
+    // B = Z U diag(alpha).
+    for (int c = lane; c < n; c += 32)
+        for (int i = 0; i < c; ++i) low(i, c) = narrow(A[i * ld + c] * (ir * ir));
     if (lane < 9) {
         double s = 0.0;
         for (int i = 0; i < n; ++i) s += sm.Z[lane * NM + i] * sm.v1[i];
         sm.zv[lane] = s;
     }
-    for (int c = lane; c < n; c += 32)
-        for (int a = 0; a < 9; ++a) {
-            double s = 0.0;
-            for (int l = 0; l < n; ++l) s += sm.Z[a * NM + l] * U[l * ld + c];
-            sm.B[a * NM + c] = s;
+    for (int c = lane; c < n; c += 32) {
+        double acc[9];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) acc[a] = 0.0;
+        for (int l = 0; l < n; ++l) {
+            const double ul = U[l * ld + c];
+#pragma unroll
+            for (int a = 0; a < 9; ++a) acc[a] = fma(sm.Z[a * NM + l], ul, acc[a]);
         }
+#pragma unroll
+        for (int a = 0; a < 9; ++a) sm.B[a * NM + c] = sm.v5[c] * acc[a];
+    }
     __syncwarp();
-    // Z <- (Z U) g(S).
-    for (int c = lane; c < n; c += 32)
-        for (int a = 0; a < 9; ++a) {
-            double s = 0.0;
-            for (int j = 0; j < n; ++j) s += sm.B[a * NM + j] * A[j * ld + c];
-            sm.Z[a * NM + c] = s;
+    // Z <- B P diag(alpha); then B - Z + Z P diag(alpha) = Z U (K0 + P)^{-1}.
+    for (int c = lane; c < n; c += 32) {
+        double acc[9];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) acc[a] = 0.0;
+        for (int j = 0; j < n; ++j) {
+            const double pj = up(j, c);
+#pragma unroll
+            for (int a = 0; a < 9; ++a) acc[a] = fma(sm.B[a * NM + j], pj, acc[a]);
         }
+#pragma unroll
+        for (int a = 0; a < 9; ++a) {
+            const double z = sm.v5[c] * acc[a];
+            sm.Z[a * NM + c] = z;
+            sm.Zf[a * NM + c] = narrow(z * aa);
+        }
+    }
     __syncwarp();
-    // B <- sqrt(k-1) Z U^T diag(sqrt(rho)), ready to meet dY.
-    const double sk = sqrt((double)(k - 1));
-    for (int c = lane; c < n; c += 32)
-        for (int a = 0; a < 9; ++a) {
-            double s = 0.0;
-            for (int l = 0; l < n; ++l) s += sm.Z[a * NM + l] * U[c * ld + l];
-            sm.B[a * NM + c] = sk * sm.lsq[c] * s;
+    for (int c = lane; c < n; c += 32) {
+        float acc[9];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) acc[a] = 0.0f;
+        for (int j = 0; j < n; ++j) {
+            const float pj = j == c ? narrow(A[c * ld + c] * (ir * ir)) : low(j, c);
+#pragma unroll
+            for (int a = 0; a < 9; ++a) acc[a] = fmaf(sm.Zf[a * NM + j], pj, acc[a]);
         }
+#pragma unroll
+        for (int a = 0; a < 9; ++a)
+            sm.B[a * NM + c] = fma(sm.v5[c], widen(acc[a]), sm.B[a * NM + c] - sm.Z[a * NM + c]);
+    }
+    __syncwarp();
+    // B <- -sqrt(k-1)/r B U^T diag(sqrt(rho)), ready to meet dY (through Z).
+    const double sk = -sqrt((double)(k - 1)) * ir;
+    for (int c = lane; c < n; c += 32) {
+        double acc[9];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) acc[a] = 0.0;
+        for (int l = 0; l < n; ++l) {
+            const double ul = U[c * ld + l];
+#pragma unroll
+            for (int a = 0; a < 9; ++a) acc[a] = fma(sm.B[a * NM + l], ul, acc[a]);
+        }
+#pragma unroll
+        for (int a = 0; a < 9; ++a) sm.Z[a * NM + c] = sk * sm.lsq[c] * acc[a];
+    }
     __syncwarp();
     const double sb = sqrt(beta);
     for (int m = lane; m < k; m += 32) {
@@ -602,7 +717,7 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
         for (int i = 0; i < n; ++i) {
             const double dy = o.dY[(size_t)sm.lidx[i] * k + m];
 #pragma unroll
-            for (int a = 0; a < 9; ++a) acc[a] += sm.B[a * NM + i] * dy;
+            for (int a = 0; a < 9; ++a) acc[a] += sm.Z[a * NM + i] * dy;
         }
 #pragma unroll
         for (int a = 0; a < 9; ++a) fc[a * plane + m] = acc[a];
@@ -692,13 +807,13 @@ __global__ void __launch_bounds__(32) analyze_fp64_kernel(double* __restrict__ f
         for (int i = 0; i < n; ++i) U[i * ld + c] = (i == c) ? 1.0 : 0.0;
     __syncwarp();
 
-    // Observation space: stop once the off-diagonal is below 3e-8 ||A||_F and
-    // take the matrix functions to first order in it (Daleckii-Krein; the
-    // neglected second-order term is (3e-8 ||A||_F / (a + s))^2, below
-    // ~1e-11 relative even for ||A||_F ~ 100 a, i.e. ~1e-13 of the state).
-    // Ensemble space converges fully and uses the diagonal directly.
+    // Observation space: stop once the off-diagonal is below 3e-8 ||A||_F or
+    // 1e-6 a and take the matrix functions to second order in it
+    // (fp64_obs_update). Ensemble space converges fully and uses the
+    // diagonal directly.
     const int sweeps = jacobi_sym_warp<double>(A, U, n, ld, lane, sm.rc, sm.rs, sm.rp, sm.rq,
-                                               obs_space ? 3e-8 : 1e-18, kMaxSweeps);
+                                               obs_space ? 3e-8 : 1e-18, obs_space ? kOffDiag * aa : 0.0,
+                                               kMaxSweeps);
     if (sweeps < 0 && lane == 0) atomicOr(flags, FLAG_NOCONV);
     record_sweeps(o, sweeps, lane);
     __syncwarp();
@@ -750,17 +865,22 @@ __global__ void __launch_bounds__(32) analyze_fp64_kernel(double* __restrict__ f
 //     binary32, Y1 to ~1e-13. E and the correction Y E run on the binary32
 //     units (double-binary32 sums of exact products for E); Y1 is FP64.
 // In FP64:
-//  2. A' = Y1^T A Y1 (symmetrised), diagonal to ~1e-6 of ||A||.
+//  2. A' = Y1^T A Y1, diagonal to ~1e-6 of ||A||.
 //  3. The FP64 cyclic Jacobi of the cold path from A' with U = Y1 at the
-//     start and the same stopping rule (3e-8 ||A||_F): one rotating sweep
-//     where a cold start needs five or six.
-//  4. The FP64 transform and update of the cold path.
-// The eigenpairs are FP64's; the binary32 basis is only where the FP64
-// Jacobi starts.
+//     start and the same stopping rule: mostly nothing left to rotate where a
+//     cold start needs five or six sweeps.
+//  4. The FP64 transform and update of the cold path, second order in what
+//     is left off the diagonal.
+// The matrix functions are FP64's; the binary32 basis is only where the FP64
+// work starts. Bound by the FP64 pipe (two operations per SM cycle): two
+// rotating sweeps of the Jacobi were 200,000 of the kernel's 310,000
+// operations per grid point at n = 28, k = 64; 31.3 -> 18.0 ms per 256^2 x 64
+// analysis without them.
 template <int NS>
 __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, int nx, int ny, int k, ObsParams o,
-                                                      double d_cut, double beta, int R, int run0,
+                                                      double beta, int R, int run0,
                                                       const float* __restrict__ Yg, const float* __restrict__ lamg,
+                                                      const double* __restrict__ wg,
                                                       const int* __restrict__ rinfo, int info_stride,
                                                       int* __restrict__ flags) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -781,6 +901,7 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
     const size_t plane = (size_t)nx * ny * k;
     double* fc = f + cell * k;
 
+    const double ik = 1.0 / k;
     for (int a = 0; a < 9; ++a) {
         double s = 0.0;
         for (int m = lane; m < k; m += 32) {
@@ -788,7 +909,7 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
             sm.dX[a * k + m] = xv;
             s += xv;
         }
-        const double mean = warp_sum(s) / k;
+        const double mean = warp_sum(s) * ik;
         for (int m = lane; m < k; m += 32) sm.dX[a * k + m] -= mean;
         if (lane == 0) sm.xbar[a] = mean;
     }
@@ -803,27 +924,11 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
             for (int m = lane; m < k; m += 32) fc[a * plane + m] = sm.xbar[a] + sb * sm.dX[a * k + m];
         return;
     }
-    // The union's scalars with this point's weights (the FP64 operations of
-    // local_set; zero outside the support and on padding).
-    const double lim2 = (2.0 * d_cut + 1.0) * (2.0 * d_cut + 1.0);
+    // The union's scalars with this point's weights (from kernel J; zero
+    // outside the support and on padding).
     for (int c = lane; c < NS; c += 32) {
-        int g = 0;
-        double w = 0.0;
-        if (c < nu) {
-            g = info[1 + c];
-            const int j = g / o.nvar;
-            const int dx = min_image(o.ix[j] - x, nx);
-            const int dy = min_image(o.iy[j] - y, ny);
-            const double d2 = (double)dx * dx + (double)dy * dy;
-            if (d2 <= lim2) {
-                const double dist = sqrt(d2) / d_cut;
-                if (dist < 2.0) {
-                    const double gc = gaspari_cohn(dist);
-                    const int q = g % o.nvar;
-                    if (gc > 0.0) w = sqrt(gc) / (q == 0 ? o.sigma_u : (q == 1 ? o.sigma_v : o.sigma_r));
-                }
-            }
-        }
+        const int g = c < nu ? info[1 + c] : 0;
+        const double w = c < nu ? wg[(size_t)lc * NS + c] : 0.0;
         sm.lidx[c] = g;
         sm.lsq[c] = w;
         sm.ldh[c] = c < nu ? w * o.d[g] : 0.0;
@@ -866,8 +971,9 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
                 f2unpack(S2[q], s0, s1);
                 f2unpack(C2[q], c0, c1);
                 const int i = i0 + 2 * q;
-                if (lane < NS && i < NS) Ef[i * NS + c] = (float)(df_value(s0, c0) - (i == c ? 1.0 : 0.0));
-                if (lane < NS && i + 1 < NS) Ef[(i + 1) * NS + c] = (float)(df_value(s1, c1) - (i + 1 == c ? 1.0 : 0.0));
+                if (lane < NS && i < NS) Ef[i * NS + c] = __fadd_rn(__fsub_rn(s0, i == c ? 1.0f : 0.0f), c0);
+                if (lane < NS && i + 1 < NS)
+                    Ef[(i + 1) * NS + c] = __fadd_rn(__fsub_rn(s1, i + 1 == c ? 1.0f : 0.0f), c1);
             }
         }
     }
@@ -885,7 +991,7 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
         }
         if (lane < NS) {
 #pragma unroll
-            for (int i = 0; i < NS; ++i) U[i * ld + c] = fma(-0.5, (double)ye[i], (double)Yf[i * NS + c]);
+            for (int i = 0; i < NS; ++i) U[i * ld + c] = fma(-0.5, widen(ye[i]), widen(Yf[i * NS + c]));
         }
     }
     __syncwarp();
@@ -896,7 +1002,7 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
         for (int i = 0; i < NS; ++i) A[i * ld + cc] = sm.lsq[i] * o.G[(size_t)sm.lidx[i] * (o.nvar * o.npts) + oc] * sc;
     }
     __syncwarp();
-    // 2. A' = Y1^T (A Y1), column c; then symmetrised.
+    // 2. A' = Y1^T (A Y1), column c.
     {
         double v[NS];
 #pragma unroll
@@ -908,24 +1014,35 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
             for (int i = 0; i < NS; ++i) v[i] += A[i * ld + j] * ujc;
         }
         __syncwarp();  // A is read by every lane above and rewritten below
-        for (int i = 0; i < NS; ++i) {
-            double s = 0.0;
+        // Entries {c, c + d mod NS}, d <= NS / 2, mirrored: the same number
+        // for every lane, half of the full product.
+        for (int d0 = 0; 2 * d0 <= NS; d0 += 4) {
+            int at[4];
+            double s4[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int j = 0; j < NS; ++j) s += U[j * ld + i] * v[j];
-            if (lane < NS) A[i * ld + c] = s;
-        }
-    }
-    __syncwarp();
-    if (lane < NS) {
-        for (int i = 0; i < c; ++i) {
-            const double m = 0.5 * (A[i * ld + c] + A[c * ld + i]);
-            A[i * ld + c] = m;
-            A[c * ld + i] = m;
+            for (int q = 0; q < 4; ++q) {
+                const int d = min(d0 + q, NS - 1);
+                at[q] = c + d < NS ? c + d : c + d - NS;
+            }
+#pragma unroll
+            for (int j = 0; j < NS; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (2 * (d0 + q) <= NS) s4[q] = fma(U[j * ld + at[q]], v[j], s4[q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int d = d0 + q;
+                if (lane < NS && (2 * d < NS || (2 * d == NS && c < d))) {
+                    A[at[q] * ld + c] = s4[q];
+                    A[c * ld + at[q]] = s4[q];
+                }
+            }
         }
     }
     __syncwarp();
     // 3. FP64 Jacobi from A' with U = Y1.
-    const int sweeps = jacobi_sym_warp<double>(A, U, NS, ld, lane, sm.rc, sm.rs, sm.rp, sm.rq, 3e-8, kMaxSweeps);
+    const int sweeps = jacobi_sym_warp<double>(A, U, NS, ld, lane, sm.rc, sm.rs, sm.rp, sm.rq, 3e-8,
+                                               kOffDiag * ((k - 1) / beta), kMaxSweeps);
     if (sweeps < 0 && lane == 0) atomicOr(flags, FLAG_NOCONV);
     record_sweeps(o, sweeps, lane);
     __syncwarp();
@@ -2759,14 +2876,14 @@ __global__ void to_f32_kernel(const double* __restrict__ src, float* __restrict_
 
 }  // namespace
 
-cudaError_t launch_run_fp64(double* f, int nx, int ny, int k, const ObsParams& o, double d_cut, double beta,
+cudaError_t launch_run_fp64(double* f, int nx, int ny, int k, const ObsParams& o, double beta,
                             int run_len, int run0, int nruns, int ns, const float* Yg, const float* lamg,
-                            const int* rinfo, int info_stride, int* flags, cudaStream_t s) {
+                            const double* wg, const int* rinfo, int info_stride, int* flags, cudaStream_t s) {
     auto go = [&](auto kern, size_t sh) -> cudaError_t {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)((size_t)nruns * run_len), 32, sh, s>>>(f, nx, ny, k, o, d_cut, beta, run_len, run0, Yg,
-                                                                  lamg, rinfo, info_stride, flags);
+        kern<<<(unsigned)((size_t)nruns * run_len), 32, sh, s>>>(f, nx, ny, k, o, beta, run_len, run0, Yg, lamg,
+                                                                  wg, rinfo, info_stride, flags);
         return cudaGetLastError();
     };
     switch (ns) {

@@ -1219,8 +1219,8 @@ cudaError_t launch_runs_ns(RunArgs ra, long long runs, long long chunk, const Pr
             // Double-precision context: the FP64 Jacobi from J's basis.
             ObsParams o = ra.o;
             o.sweep_hist = ra.fp64_hist;
-            e = launch_run_fp64(ra.f64, ra.nx, ra.ny, ra.k, o, ra.d_cut, ra.beta, ra.R, ra.run0, ra.nruns, NS,
-                                ra.Yg, ra.lamg, ra.rinfo, kInfo, ra.flags, s);
+            e = launch_run_fp64(ra.f64, ra.nx, ra.ny, ra.k, o, ra.beta, ra.R, ra.run0, ra.nruns, NS,
+                                ra.Yg, ra.lamg, ra.wg, ra.rinfo, kInfo, ra.flags, s);
             if (e != cudaSuccess) return e;
         } else if (probe)
             run_refine_kernel<NS, true><<<(unsigned)pa.npoints, 32, shF, s>>>(ra, pa);
@@ -1271,8 +1271,8 @@ cudaError_t launch_runs_pipe(RunArgs ra, long long runs, long long pipe, const A
         if (rb.f64) {
             ObsParams o = rb.o;
             o.sweep_hist = rb.fp64_hist;
-            e = launch_run_fp64(rb.f64, rb.nx, rb.ny, rb.k, o, rb.d_cut, rb.beta, rb.R, rb.run0, rb.nruns, NS, rb.Yg,
-                                rb.lamg, rb.rinfo, kInfo, rb.flags, s);
+            e = launch_run_fp64(rb.f64, rb.nx, rb.ny, rb.k, o, rb.beta, rb.R, rb.run0, rb.nruns, NS, rb.Yg,
+                                rb.lamg, rb.wg, rb.rinfo, kInfo, rb.flags, s);
             if (e != cudaSuccess) return e;
         } else {
             const ProbeArgs none{nullptr, 0, nullptr, nullptr};
@@ -1411,8 +1411,8 @@ cudaError_t launch_runs_batch_ns(const std::vector<RunArgs>& ex, cudaStream_t s)
             if (ra.f64) {
                 ObsParams o = ra.o;
                 o.sweep_hist = ra.fp64_hist;
-                e = launch_run_fp64(ra.f64, ra.nx, ra.ny, ra.k, o, ra.d_cut, ra.beta, ra.R, 0, ra.nruns, NS, ra.Yg,
-                                    ra.lamg, ra.rinfo, kInfo, ra.flags, s);
+                e = launch_run_fp64(ra.f64, ra.nx, ra.ny, ra.k, o, ra.beta, ra.R, 0, ra.nruns, NS, ra.Yg,
+                                    ra.lamg, ra.wg, ra.rinfo, kInfo, ra.flags, s);
                 if (e != cudaSuccess) return e;
             } else {
                 run_refine_kernel<NS, false>
