@@ -59,6 +59,7 @@ struct lbm_ctx {
     int prod = PROD_FP64;  // ensemble-space Gram arithmetic (mixed precision)
     int run_pipe = 0;      // runs per pipelined chunk of the run analysis (0: not pipelined)
     int run_batched = 1;   // in a batch: run analysis in the batched launches (0: launched on its own)
+    cudaMemPool_t pool = nullptr;  // the context's stream-ordered scratch
     int* sweep_hist = nullptr;  // [32] Jacobi sweeps per point (diagnostic)
     bool sweep_stats = false;
     bool observed = false;
@@ -312,20 +313,45 @@ int observe_impl(lbm_ctx* c, int npts, const int* ix, const int* iy, const doubl
     return LBM_OK;
 }
 
-// Device buffers of one misfit/gradient call, allocated and released in
-// stream order on the context stream.
+// Stream-ordered scratch comes from a pool of the context's own that keeps up
+// to kPoolKeep bytes between calls (given back at lbm_destroy): the device's
+// default pool returns everything at each synchronisation, and mapping the
+// 5 GB of a 256^2 x 64 gradient anew took 8 of its 56 ms.
+constexpr unsigned long long kPoolKeep = 16ull << 30;
+
+cudaError_t scratch_pool(lbm_ctx* c) {
+    if (c->pool) return cudaSuccess;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    cudaError_t e = cudaGetDevice(&props.location.id);
+    if (e != cudaSuccess) return e;
+    cudaMemPool_t pool = nullptr;
+    if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+    unsigned long long keep = kPoolKeep;
+    if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) {
+        cudaMemPoolDestroy(pool);
+        return e;
+    }
+    c->pool = pool;
+    return cudaSuccess;
+}
+
+// Device buffers of one call, allocated and released in stream order on the
+// context stream.
 struct StreamScratch {
-    cudaStream_t s;
+    lbm_ctx* c;
     std::vector<void*> bufs;
-    explicit StreamScratch(cudaStream_t st) : s(st) {}
+    explicit StreamScratch(lbm_ctx* ctx) : c(ctx) {}
     cudaError_t get(void** p, size_t bytes) {
         *p = nullptr;
-        cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, s);
+        cudaError_t e = scratch_pool(c);
+        if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, c->pool, c->stream);
         if (e == cudaSuccess) bufs.push_back(*p);
         return e;
     }
     ~StreamScratch() {
-        for (void* b : bufs) cudaFreeAsync(b, s);
+        for (void* b : bufs) cudaFreeAsync(b, c->stream);
     }
 };
 
@@ -372,7 +398,7 @@ int misfit_impl(lbm_ctx* c, const lbm_window* win, const double* w, double* J, d
                     : launch_lbm_step_f64((const double*)in, (double*)out,
                                           (const double*)c->force, p, c->flags, c->stream);
     };
-    StreamScratch sc(c->stream);
+    StreamScratch sc(c);
     const int nck = want_grad ? (N + C - 1) / C : 0;
     const int nseg = want_grad ? std::min(C, N) - 1 : 0;
     std::vector<void*> ck(nck), seg(nseg);
@@ -425,8 +451,10 @@ int misfit_impl(lbm_ctx* c, const lbm_window* win, const double* w, double* J, d
     if (want_grad) {
         CK(c, cudaMemcpyAsync(ck[0], prev, S, cudaMemcpyDeviceToDevice, c->stream), "checkpoint");
     }
+    // The last segment's states stay where the reverse sweep wants them first.
+    const int last = want_grad ? (nck - 1) * C : N;
     for (int t = 1; t <= N; ++t) {
-        void* out = (want_grad && t % C == 0 && t < N) ? ck[t / C] : tmp[t & 1];
+        void* out = (want_grad && t % C == 0 && t < N) ? ck[t / C] : (t > last && t < N ? seg[t - last - 1] : tmp[t & 1]);
         CK(c, step(prev, out), "launching LBM step");
         const int r = obs_time(t);
         if (r >= 0)
@@ -460,7 +488,7 @@ int misfit_impl(lbm_ctx* c, const lbm_window* win, const double* w, double* J, d
             const int t0 = sgi * C, t1 = std::min(t0 + C, N);
             st[0] = ck[sgi];
             for (int i = 1; i < t1 - t0; ++i) {
-                CK(c, step(st[i - 1], seg[i - 1]), "launching LBM step");
+                if (t0 != last) CK(c, step(st[i - 1], seg[i - 1]), "launching LBM step");
                 st[i] = seg[i - 1];
             }
             for (int t = t1 - 1; t >= t0; --t) {
@@ -799,7 +827,7 @@ int lbm_velocity_rmse(lbm_ctx* c, lbm_ctx* truth, double* rmse, int ptr_kind) {
         cudaEventDestroy(ev);
         CK(c, e, "ordering the two streams");
     }
-    StreamScratch sc(c->stream);
+    StreamScratch sc(c);
     void* buf;
     CK(c, sc.get(&buf, (4 * n + rmse_work_doubles() + 1) * sizeof(double)), "allocating RMSE scratch");
     double* b = (double*)buf;
@@ -825,10 +853,9 @@ int lbm_energy_spectrum(lbm_ctx* c, double* E, int nshells, int ptr_kind) {
     const int nsh = nshells < all ? nshells : all;
     const size_t work = spectrum_work_bytes(c->nx, c->ny, c->k, nsh);
     const size_t out = ptr_kind == LBM_PTR_HOST ? (size_t)nshells * sizeof(double) : 0;
+    StreamScratch sc(c);
     void* buf = nullptr;
-    // Stream-ordered scratch: the diagnostic is occasional and its buffers
-    // (about 1 KiB per member and lattice row) are returned right after.
-    CK(c, cudaMallocAsync(&buf, work + out, c->stream), "allocating spectrum scratch");
+    CK(c, sc.get(&buf, work + out), "allocating spectrum scratch");
     double* Ed = ptr_kind == LBM_PTR_HOST
                      ? reinterpret_cast<double*>(static_cast<unsigned char*>(buf) + work)
                      : E;
@@ -838,11 +865,9 @@ int lbm_energy_spectrum(lbm_ctx* c, double* E, int nshells, int ptr_kind) {
         e = cudaMemsetAsync(Ed + nsh, 0, (size_t)(nshells - nsh) * sizeof(double), c->stream);
     if (e == cudaSuccess && ptr_kind == LBM_PTR_HOST)
         e = cudaMemcpyAsync(E, Ed, out, cudaMemcpyDeviceToHost, c->stream);
-    const cudaError_t e2 = cudaFreeAsync(buf, c->stream);
     if (e == cudaErrorInvalidValue)
         return fail(c, LBM_EINVAL, "lattice too large for the spectrum diagnostic's shared memory");
     CK(c, e, "launching the energy spectrum");
-    CK(c, e2, "freeing spectrum scratch");
     return ptr_kind == LBM_PTR_HOST ? read_flags(c) : LBM_OK;
 }
 
@@ -944,7 +969,7 @@ int letkf_probe_transform(lbm_ctx* c, double d_cut, double beta, int npoints, co
         return fail(c, LBM_EINVAL,
                     "the transform probe needs the run analysis (run length > 0, every grid point with p < members, "
                     "unions of at most 32 scalars)");
-    StreamScratch sc(c->stream);
+    StreamScratch sc(c);
     void *d_cells, *d_work, *d_T = T;
     const size_t tbytes = (size_t)npoints * c->k * c->k * sizeof(double);
     CK(c, sc.get(&d_cells, (size_t)npoints * sizeof(int)), "allocating probe points");
@@ -1062,6 +1087,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->ana_scratch);
     cudaFree(c->nudge_obs);
     cudaFree(c->sweep_hist);
+    if (c->pool) cudaMemPoolDestroy(c->pool);
     if (c->aux_ready) {
         cudaStreamSynchronize(c->aux.s2);
         cudaEventDestroy(c->aux.start);
