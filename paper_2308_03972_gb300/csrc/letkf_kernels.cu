@@ -1428,7 +1428,7 @@ __host__ __device__ inline MixScratch mix_scratch_at(void* base, long long chunk
     m.lsq = reinterpret_cast<double*>(p);
     p += (size_t)chunk * nobs * sizeof(double);
     m.lidx = reinterpret_cast<int*>(p);
-    p += (size_t)chunk * nobs * sizeof(int);
+    p += ((size_t)chunk * nobs * sizeof(int) + 15) / 16 * 16;  // the Gram and b after it need 8 bytes
     m.pcount = reinterpret_cast<int*>(p);
     p += ((size_t)chunk * sizeof(int) + 15) / 16 * 16;
     m.C32 = (kg && gsz == 4) ? reinterpret_cast<float*>(p) : nullptr;
@@ -1445,7 +1445,7 @@ __host__ __device__ inline MixScratch mix_scratch_at(void* base, long long chunk
 // Bytes of one scratch buffer, rounded up to 256 so that the second buffer of
 // the pair starts as aligned as the first (its FP64 arrays need 8 bytes).
 __host__ __device__ inline size_t mix_buf_bytes(long long chunk, int nobs, int nm, int kg, int gsz) {
-    return ((size_t)chunk * mix_scratch_bytes_per_point(nobs, nm, kg, gsz) + 16 + 255) / 256 * 256;
+    return ((size_t)chunk * mix_scratch_bytes_per_point(nobs, nm, kg, gsz) + 32 + 255) / 256 * 256;
 }
 
 // ---- Local Gram matrices in reduced precision (ensemble-space form) --------
