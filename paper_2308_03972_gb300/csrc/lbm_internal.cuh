@@ -60,6 +60,9 @@ struct ObsParams {
     int plmax = 0;     // capacity of one grid point's local list (0: nobs); a
                        // point with more local scalars is reported too large
     int* sweep_hist = nullptr;  // [32] Jacobi sweep counts per point, or null
+    // Localisation weights by squared distance (an integer), or null: per
+    // distance G and sqrt(G) / sigma of u, v, rho, all zero outside the support.
+    const double* wtab = nullptr;
 };
 
 // ---- lbm_kernels.cu -------------------------------------------------------
@@ -138,6 +141,15 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
 
 // dst = (float) src, n elements.
 cudaError_t launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t s);
+
+// ObsParams::wtab: one entry per squared distance replaces the FP64 square
+// roots, divisions and polynomials of every (grid point, observation) pair
+// (FP64 issues at 1/64 of the binary32 rate). weight_table_bytes: capacity
+// for a lattice (up to 8 MB); entries: used for d_cut, 0 where the capacity
+// does not hold them (the kernels then evaluate the weights themselves).
+size_t weight_table_bytes(int nx, int ny);
+int weight_table_entries(int nx, int ny, double d_cut);
+cudaError_t launch_weight_table(const ObsParams& o, double d_cut, int entries, double* tab, cudaStream_t s);
 
 // ---- letkf_runs.cu --------------------------------------------------------
 // Mixed-precision analysis over runs of run_len consecutive grid points of a

@@ -35,6 +35,7 @@ struct lbm_ctx {
     float* dY32 = nullptr; // [nobs][k] binary32 copy (mixed precision)
     void* ana_scratch = nullptr;   // analysis scratch (mixed precision)
     size_t ana_scratch_bytes = 0;
+    double* wtab = nullptr;        // localisation weights by squared distance
     // Observation geometry of the last letkf_observe, and the largest local
     // problem it gives for a cached d_cut.
     std::vector<int> geo_ix, geo_iy;
@@ -571,6 +572,9 @@ int analyze_prepare(lbm_ctx* c, double d_cut, double beta, AnalysisPlan* plan, b
         CK(c, cudaMalloc(&c->ana_scratch, scratch), "allocating analysis scratch");
         c->ana_scratch_bytes = scratch;
     }
+    // Sized by the lattice, so a captured analysis keeps its address.
+    if (!c->wtab)
+        CK(c, cudaMalloc(&c->wtab, weight_table_bytes(c->nx, c->ny)), "allocating weight table");
     if ((is_fp32(c) || run_len > 0) && !c->aux_ready) {
         CK(c, cudaStreamCreateWithFlags(&c->aux.s2, cudaStreamNonBlocking), "creating stream");
         CK(c, cudaEventCreateWithFlags(&c->aux.start, cudaEventDisableTiming), "creating event");
@@ -587,12 +591,20 @@ int analyze_prepare(lbm_ctx* c, double d_cut, double beta, AnalysisPlan* plan, b
 ObsParams obs_params(lbm_ctx* c, const AnalysisPlan& pl) {
     return ObsParams{c->npts, c->ix,    c->iy,   c->dY,       c->d,
                      c->G,    c->sigma_u, c->sigma_v, c->dY32, c->nvar,
-                     c->sigma_r, pl.plmax, c->sweep_stats ? c->sweep_hist : nullptr};
+                     c->sigma_r, pl.plmax, c->sweep_stats ? c->sweep_hist : nullptr,
+                     weight_table_entries(c->nx, c->ny, pl.d_cut) ? c->wtab : nullptr};
+}
+
+// Fills the weight table of an analysis on stream s, before its kernels.
+cudaError_t fill_weights(const lbm_ctx* c, const ObsParams& o, const AnalysisPlan& pl, cudaStream_t s) {
+    return o.wtab ? launch_weight_table(o, pl.d_cut, weight_table_entries(c->nx, c->ny, pl.d_cut), c->wtab, s)
+                  : cudaSuccess;
 }
 
 // Device part: the analysis kernels on the context stream (capturable).
 int analyze_launch(lbm_ctx* c, const AnalysisPlan& pl) {
     const ObsParams o = obs_params(c, pl);
+    CK(c, fill_weights(c, o, pl, c->stream), "launching weight table");
     if (pl.run_len > 0) {
         const AnalyzeAux* aux = c->aux_ready ? &c->aux : nullptr;
         if (is_fp32(c))
@@ -1085,6 +1097,7 @@ void lbm_destroy(lbm_ctx* c) {
     cudaFree(c->flags);
     cudaFree(c->stage);
     cudaFree(c->ana_scratch);
+    cudaFree(c->wtab);
     cudaFree(c->nudge_obs);
     cudaFree(c->sweep_hist);
     if (c->pool) cudaMemPoolDestroy(c->pool);
@@ -1207,6 +1220,7 @@ int batch_analyze(lbm_batch* b, const std::vector<AnalysisPlan>& plans, const st
         const AnalysisPlan& pl = plans[i];
         if (pl.run_len > 0 && c->run_batched) {
             const bool f32 = is_fp32(c);
+            BK(b, fill_weights(c, obs_params(c, pl), pl, s), "launching weight table");
             items.push_back(RunItem{f32 ? (float*)c->f[c->cur] : nullptr, f32 ? nullptr : (double*)c->f[c->cur],
                                     c->nx, c->ny, c->k, pl.run_len, pl.maxunion, obs_params(c, pl), pl.d_cut,
                                     pl.beta, c->flags, c->ana_scratch});

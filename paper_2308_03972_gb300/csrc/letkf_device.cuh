@@ -4,6 +4,8 @@
 #include <cmath>
 #include <cstdint>
 
+#include "lbm_internal.cuh"
+
 namespace lbmgpu {
 namespace {
 
@@ -43,6 +45,27 @@ __device__ __forceinline__ double gaspari_cohn(double d) {
         return d * d * (5.0 / 3.0 + d * (0.625 + d * (-0.5 + d * (1.0 / 12.0)))) - 5.0 * d + 4.0 -
                (2.0 / 3.0) / d;
     return 0.0;
+}
+
+// Localisation weight at squared distance d2 <= support_lim2(d_cut): G
+// (col 0) or sqrt(G) / sigma of scalar col - 1; 0 outside the support
+// (r / d_cut < 2 and G > 0 decide, in FP64).
+__device__ __forceinline__ double weight_eval(const ObsParams& o, long long d2, double d_cut, int col) {
+    const double dist = sqrt((double)d2) / d_cut;
+    if (!(dist < 2.0)) return 0.0;
+    const double g = gaspari_cohn(dist);
+    if (!(g > 0.0)) return 0.0;
+    return col == 0 ? g : sqrt(g) / (col == 1 ? o.sigma_u : (col == 2 ? o.sigma_v : o.sigma_r));
+}
+__device__ __forceinline__ double weight_of(const ObsParams& o, long long d2, double d_cut, int col) {
+    return o.wtab ? __ldg(o.wtab + 4 * d2 + col) : weight_eval(o, d2, d_cut, col);
+}
+// The same for observation point j seen from grid point (x, y); lim2 =
+// support_lim2(d_cut).
+__device__ __forceinline__ double point_weight(const ObsParams& o, int j, int x, int y, int nx, int ny, double d_cut,
+                                               long long lim2, int col) {
+    const long long d2 = dist2(min_image(o.ix[j] - x, nx), min_image(o.iy[j] - y, ny));
+    return d2 > lim2 ? 0.0 : weight_of(o, d2, d_cut, col);
 }
 
 // ---- Double-binary32 arithmetic -------------------------------------------

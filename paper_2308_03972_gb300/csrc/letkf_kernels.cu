@@ -120,35 +120,26 @@ __device__ int local_set(const ObsParams& o, int x, int y, int nx, int ny, doubl
     for (int j0 = 0; j0 < o.npts; j0 += 32) {
         const int j = j0 + lane;
         bool in = false;
-        double g = 0.0;
+        long long d2 = 0;
         if (j < o.npts) {
-            const int dx = min_image(o.ix[j] - x, nx);
-            const int dy = min_image(o.iy[j] - y, ny);
+            d2 = dist2(min_image(o.ix[j] - x, nx), min_image(o.iy[j] - y, ny));
             // Integer prefilter well outside the support (r > 2 d_cut + 1);
             // the decision itself is r / d_cut < 2 in FP64.
-            if (dist2(dx, dy) <= lim2) {
-                const double d2 = (double)dx * dx + (double)dy * dy;
-                const double dist = sqrt(d2) / d_cut;
-                if (dist < 2.0) {
-                    g = gaspari_cohn(dist);
-                    in = g > 0.0;
-                }
-            }
+            if (d2 <= lim2) in = weight_of(o, d2, d_cut, 0) > 0.0;
         }
         const unsigned bal = __ballot_sync(kFull, in);
         if (in) {
             const int pos = o.nvar * (count + __popc(bal & ((1u << lane) - 1u)));
-            const double sg = sqrt(g);
             // Entries past the capacity are counted, not stored; the caller
             // reports the point as too large.
             if (pos + o.nvar <= cap) {
                 lidx[pos] = o.nvar * j;
                 lidx[pos + 1] = o.nvar * j + 1;
-                lsq[pos] = sg / o.sigma_u;
-                lsq[pos + 1] = sg / o.sigma_v;
+                lsq[pos] = weight_of(o, d2, d_cut, 1);
+                lsq[pos + 1] = weight_of(o, d2, d_cut, 2);
                 if (o.nvar == 3) {
                     lidx[pos + 2] = 3 * j + 2;
-                    lsq[pos + 2] = sg / o.sigma_r;
+                    lsq[pos + 2] = weight_of(o, d2, d_cut, 3);
                 }
             }
         }
@@ -1466,20 +1457,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// sqrt(G(r / d_cut)) of observation point j seen from (x, y), 0 outside the
-// support: the same FP64 operations as local_set.
-__device__ __forceinline__ double local_weight(const ObsParams& o, int j, int x, int y, int nx,
-                                               int ny, double d_cut, long long lim2) {
-    const int dx = min_image(o.ix[j] - x, nx);
-    const int dy = min_image(o.iy[j] - y, ny);
-    if (dist2(dx, dy) > lim2) return 0.0;  // lim2 = support_lim2(d_cut)
-    const double d2 = (double)dx * dx + (double)dy * dy;
-    const double dist = sqrt(d2) / d_cut;
-    if (!(dist < 2.0)) return 0.0;
-    const double g = gaspari_cohn(dist);
-    return g > 0.0 ? sqrt(g) : 0.0;
-}
-
 // Merged local sets of the kGramPts grid points cell0 + li0 + q (q < kGramPts,
 // li0 + q < ncell), in increasing point order, into U; pcnt[q] counts the
 // local points of grid point q. Returns the merged count. Block-cooperative
@@ -1498,7 +1475,7 @@ __device__ int gram_merge(const ObsParams& o, int nx, int ny, double d_cut, int 
             for (int q = 0; q < kGramPts; ++q) {
                 if (li0 + q >= ncell) break;
                 const int cell = cell0 + li0 + q;
-                if (local_weight(o, j, cell % nx, cell / nx, nx, ny, d_cut, lim2) > 0.0) bits |= 1u << q;
+                if (point_weight(o, j, cell % nx, cell / nx, nx, ny, d_cut, lim2, 0) > 0.0) bits |= 1u << q;
             }
         }
         const bool in = bits != 0u;
@@ -1578,9 +1555,9 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_kernel(int nx, in
                 float wv = 0.0f;
                 if (r < rows && li0 + q < ncell) {
                     const int cell = cell0 + li0 + q;
-                    const double sg = local_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2);
                     const int qv = r % nv;
-                    const double l = sg / (qv == 0 ? o.sigma_u : (qv == 1 ? o.sigma_v : o.sigma_r));
+                    const double l =
+                        point_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2, 1 + qv);
                     wv = (float)(l * l);
                 }
                 Ws[q][rr] = wv;
@@ -1775,9 +1752,9 @@ __global__ void __launch_bounds__(32 * kGramPts, 1)
                 float wv = 0.0f;
                 if (rr < nr && li0 + q < ncell) {
                     const int cell = cell0 + li0 + q;
-                    const double sg = local_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2);
                     const int qv = r % nv;
-                    const double l = sg / (qv == 0 ? o.sigma_u : (qv == 1 ? o.sigma_v : o.sigma_r));
+                    const double l =
+                        point_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2, 1 + qv);
                     wv = (float)(l * l);
                 }
                 Ws[q * kTcKC + rr] = wv;
@@ -1939,7 +1916,6 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_fp64_kernel(int n
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int li0 = blockIdx.x * kGramPts;
     const int nv = o.nvar;
-    const double sig[3] = {o.sigma_u, o.sigma_v, o.sigma_r};
     const int total = gram_merge(o, nx, ny, d_cut, cell0, li0, ncell, U, pcnt, wcount);
     const long long lim2 = support_lim2(d_cut);
     bool any_ens = false;
@@ -1968,8 +1944,8 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_fp64_kernel(int n
                 double wv = 0.0;
                 if (r < rows && li0 + q < ncell) {
                     const int cell = cell0 + li0 + q;
-                    const double sg = local_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2);
-                    const double l = sg / sig[r % nv];
+                    const double l =
+                        point_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2, 1 + r % nv);
                     wv = l * l;
                 }
                 Ws[q][rr] = wv;
@@ -2101,9 +2077,9 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_df_kernel(int nx,
                 double wv = 0.0, dv = 0.0;
                 if (r < rows && li0 + q < ncell) {
                     const int cell = cell0 + li0 + q;
-                    const double sg = local_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2);
                     const int qv = r % nv;
-                    const double l = sg / (qv == 0 ? o.sigma_u : (qv == 1 ? o.sigma_v : o.sigma_r));
+                    const double l =
+                        point_weight(o, U[r / nv], cell % nx, cell / nx, nx, ny, d_cut, lim2, 1 + qv);
                     wv = l * l;
                     dv = o.d[nv * U[r / nv] + qv];
                 }
@@ -2287,7 +2263,7 @@ __host__ __device__ inline size_t jacobi_block_smem_bytes(int nm) {
            4 * sizeof(unsigned) + (kBlkThreads / 32) * sizeof(float) + sizeof(int);
 }
 
-__global__ void __launch_bounds__(kBlkThreads) mixed_jacobi_block_kernel(int nx, int ny, int k, ObsParams o,
+__global__ void __launch_bounds__(kBlkThreads, 5) mixed_jacobi_block_kernel(int nx, int ny, int k, ObsParams o,
                                                                          double d_cut, double beta,
                                                                          int cell0, int nm, MixScratch sc,
                                                                          int* __restrict__ flags) {
@@ -2869,12 +2845,40 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
     }
 }
 
+__global__ void weight_table_kernel(ObsParams o, double d_cut, int n, double* __restrict__ tab) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) tab[i] = weight_eval(o, i >> 2, d_cut, i & 3);
+}
+
 __global__ void to_f32_kernel(const double* __restrict__ src, float* __restrict__ dst, size_t n) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dst[i] = (float)src[i];
 }
 
 }  // namespace
+
+// Squared distances on the lattice: 0 .. d2max.
+static long long lattice_d2max(int nx, int ny) {
+    return (long long)(nx / 2) * (nx / 2) + (long long)(ny / 2) * (ny / 2);
+}
+constexpr long long kWeightEntries = 1 << 18;
+
+size_t weight_table_bytes(int nx, int ny) {
+    const long long n = lattice_d2max(nx, ny) + 1;
+    return (size_t)(n < kWeightEntries ? n : kWeightEntries) * 4 * sizeof(double);
+}
+
+int weight_table_entries(int nx, int ny, double d_cut) {
+    const long long d2max = lattice_d2max(nx, ny), lim2 = support_lim2(d_cut);
+    const long long last = lim2 < d2max ? lim2 : d2max;
+    return last < kWeightEntries ? (int)last + 1 : 0;
+}
+
+cudaError_t launch_weight_table(const ObsParams& o, double d_cut, int entries, double* tab, cudaStream_t s) {
+    const int n = 4 * entries;
+    weight_table_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(o, d_cut, n, tab);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_run_fp64(double* f, int nx, int ny, int k, const ObsParams& o, double beta,
                             int run_len, int run0, int nruns, int ns, const float* Yg, const float* lamg,

@@ -137,17 +137,7 @@ __device__ __forceinline__ float pick_reg(const float (&a)[NS], int idx) {
 // (x, y): the local-set test of the other analysis kernels (FP64, the same
 // operations), zero outside the support.
 __device__ __forceinline__ double obs_weight(const RunArgs& ra, int j, int q, int x, int y) {
-    const ObsParams& o = ra.o;
-    const int dx = min_image(o.ix[j] - x, ra.nx);
-    const int dy = min_image(o.iy[j] - y, ra.ny);
-    if (dist2(dx, dy) > ra.lim2) return 0.0;
-    const double d2 = (double)dx * dx + (double)dy * dy;
-    const double dist = sqrt(d2) / ra.d_cut;
-    if (!(dist < 2.0)) return 0.0;
-    const double g = gaspari_cohn(dist);
-    if (!(g > 0.0)) return 0.0;
-    const double sig = q == 0 ? o.sigma_u : (q == 1 ? o.sigma_v : o.sigma_r);
-    return sqrt(g) / sig;
+    return point_weight(ra.o, j, x, y, ra.nx, ra.ny, ra.d_cut, ra.lim2, 1 + q);
 }
 
 // ---- per-run union of the local sets --------------------------------------
