@@ -1987,21 +1987,6 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_fp64_kernel(int n
         if (lane + 32 * c < k) sc.b64[(size_t)li * k + lane + 32 * c] = bacc[c];
 }
 
-// A double-binary32 sum (s, c), plus (ah + al) when diag, renormalised into
-// binary32 high and low halves (Fast2Sum: the compensated sum's s dominates).
-__device__ __forceinline__ void df_pair_out(float s, float c, bool diag, float ah, float al, float& hi,
-                                            float& lo) {
-    if (diag) {
-        float t, e;
-        two_sum(s, ah, t, e);
-        c = __fadd_rn(c, __fadd_rn(e, al));
-        s = t;
-    }
-    const float h = __fadd_rn(s, c);
-    hi = h;
-    lo = __fsub_rn(c, __fsub_rn(h, s));
-}
-
 // Double-binary32 Gram (PROD_DF32, the default of a mixed-precision
 // context): the C and b of the FP64 Gram pass to FP64-class accuracy on the
 // binary32 units. The staged rows are split once into binary32 halves
@@ -2956,9 +2941,7 @@ static cudaError_t launch_gram_mode(int nx, int ny, int k, const ObsParams& o, d
         if (k <= 64) return go(local_gram_fp64_kernel<64>);
         return go(local_gram_fp64_kernel<128>);
     } else if constexpr (MODE == PROD_DF32) {
-        if (k <= 16) return go(local_gram_df_kernel<16>);
-        if (k <= 32) return go(local_gram_df_kernel<32>);
-        if (k <= 64) return go(local_gram_df_kernel<64>);
+        if (k <= 64) return go(local_gram_df_kernel<64>);  // k > kOuterMaxK
         return go(local_gram_df_kernel<128>);
     } else {
         if (k <= 16) return go(local_gram_kernel<16>);
@@ -3033,13 +3016,24 @@ static cudaError_t launch_gram(int prod, int nx, int ny, int k, const ObsParams&
     return launch_gram_tc<false>(nx, ny, k, o, d_cut, aa, cell0, nc, sc, flags, s);
 }
 
-size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int nmax, int k, int prod) {
+// Whether the double-binary32 Gram goes through the points' outer products:
+// up to kOuterMaxK members. Above, the rows themselves are multiplied
+// (local_gram_df_kernel): the other form's C differs from this one's at 1e-13,
+// which changes the binary32 matrix that kernel (A) starts from at 0.4% of
+// the grid points at k = 64, and the binary32 transform of such a point then
+// differs by up to three units in the last place (up to one for k <= 32).
+static bool gram_by_outer(int npts, int kg, int prod) {
+    return kg && kg <= kOuterMaxK && prod == PROD_DF32 && npts > 0;
+}
+
+size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int npts, int nmax, int k, int prod) {
     if (!fp32) return 0;
     const int nm = mixed_nm(nmax);
     const int kg = gram_k(fp32, k, prod), gsz = gram_sz(prod);
     const long long cells = (long long)nx * ny;
     const long long chunk = mix_chunk(cells, nl, nm, kg, gsz);
-    return (chunk < cells ? 2 : 1) * mix_buf_bytes(chunk, nl, nm, kg, gsz);  // double-buffered
+    return (chunk < cells ? 2 : 1) * mix_buf_bytes(chunk, nl, nm, kg, gsz) +  // double-buffered
+           (gram_by_outer(npts, kg, prod) ? gram_outer_bytes(npts, kg) : 0);
 }
 
 cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsParams& o,
@@ -3089,6 +3083,12 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         // scratch is double-buffered, (A) of chunk c waits for (B) of c-2.
         if ((e = cudaEventRecord(aux->start, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(aux->s2, aux->start, 0)) != cudaSuccess) return e;
+        const bool outer = gram_by_outer(o.npts, kg, prod);
+        GramArgs ga{nx, ny, k, o, d_cut};
+        if (outer) {
+            gram_outer_at((unsigned char*)scratch + (chunk < cells ? 2 : 1) * buf_bytes, o.npts, k, &ga);
+            if ((e = launch_outer(ga, aux->s2)) != cudaSuccess) return e;
+        }
         int c = 0;
         for (long long c0 = 0; c0 < cells; c0 += chunk, ++c) {
             const int nc = (int)((cells - c0) < chunk ? (cells - c0) : chunk);
@@ -3097,7 +3097,14 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
             if (prod == PROD_DF32) sc = mix_scratch_df2(sc, chunk, kg);
             if (c >= 2 && (e = cudaStreamWaitEvent(aux->s2, aux->ref_done[b], 0)) != cudaSuccess)
                 return e;
-            if (kg && (e = launch_gram(prod, nx, ny, k, o, d_cut, (k - 1) / beta, (int)c0, nc, sc, flags,
+            if (outer) {
+                ga.cell0 = (int)c0;
+                ga.ncell = nc;
+                ga.C32 = sc.C32;
+                ga.Clo = sc.Clo;
+                ga.b64 = sc.b64;
+                if ((e = launch_gram_outer(ga, (k - 1) / beta, aux->s2)) != cudaSuccess) return e;
+            } else if (kg && (e = launch_gram(prod, nx, ny, k, o, d_cut, (k - 1) / beta, (int)c0, nc, sc, flags,
                                        aux->s2)) != cudaSuccess)
                 return e;
             if (nm <= NREG && runA > 1)
