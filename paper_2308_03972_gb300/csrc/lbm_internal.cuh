@@ -174,6 +174,29 @@ void gram_outer_at(void* base, int npts, int k, GramArgs* g);
 cudaError_t launch_outer(const GramArgs& g, cudaStream_t s);
 cudaError_t launch_gram_outer(const GramArgs& g, double aa, cudaStream_t s);
 
+// ---- letkf_wide.cu --------------------------------------------------------
+// Refinement and update (kernel (B)) of the grid points cell0 .. of a chunk
+// with local problems up to nm, 32 < nm <= 128, from kernel (A)'s basis X
+// [.][xr][xr], local lists lsq, lidx and counts pcount, and the Gram pass's C
+// (C32 with or without Clo, or C64) and b (b32 or b64).
+struct WideArgs {
+    float* f;
+    int nx, ny, k;
+    ObsParams o;
+    double d_cut, beta;
+    int cell0, nm;
+    const float* X;
+    int xr;
+    const double* lsq;
+    const int *lidx, *pcount;
+    const float *C32, *Clo;
+    const double* C64;
+    const float* b32;
+    const double* b64;
+    int* flags;
+};
+cudaError_t launch_analyze_wide(const WideArgs& a, int ncell, cudaStream_t s);
+
 // ---- letkf_runs.cu --------------------------------------------------------
 // Mixed-precision analysis over runs of run_len consecutive grid points of a
 // row (one warp each; warm-started binary32 Jacobi over the union of the

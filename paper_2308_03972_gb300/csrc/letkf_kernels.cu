@@ -2241,8 +2241,6 @@ __global__ void __launch_bounds__(32 * kJacWarps, 4) mixed_jacobi_run_kernel(int
 // Kernel (A) for local problems of 33..128: the binary32 Jacobi of
 // jacobi_sym_block, kBlkThreads threads per grid point, same output.
 constexpr int kBlkThreads = 256;
-constexpr int kWideWarps = 4;  // warps per grid point of kernel (B) above NREG
-
 __host__ __device__ inline size_t jacobi_block_smem_bytes(int nm) {
     return 2 * (size_t)nm * (nm + 1) * sizeof(float) + 64 * (2 * sizeof(float) + 2 * sizeof(int)) +
            4 * sizeof(unsigned) + (kBlkThreads / 32) * sizeof(float) + sizeof(int);
@@ -3050,14 +3048,13 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         to_f32_kernel<<<(unsigned)((nd + 255) / 256), 256, 0, s>>>(o.dY, o.dY32, nd);
         const int cap = o.plmax > 0 ? o.plmax : nobs;
         const size_t shB = mix_smem_bytes(k, cap, nm);
-        const bool wide = nm > NREG, big = nm > NMID;
+        const bool wide = nm > NREG;
         const size_t shA = wide ? jacobi_block_smem_bytes(nm) : 0;
-        // Above NREG a grid point has kWideWarps warps in kernel (B).
-        auto kernB = big ? analyze_mixed_kernel<true, true, kWideWarps>
-                         : (wide ? analyze_mixed_kernel<true, false, kWideWarps> : analyze_mixed_kernel<false, false, 1>);
-        const int thB = wide ? 32 * kWideWarps : 32;
-        e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
-        if (e != cudaSuccess) return e;
+        const auto kernB = analyze_mixed_kernel<false, false, 1>;
+        if (!wide) {
+            e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
+            if (e != cudaSuccess) return e;
+        }
         if (wide) {
             e = cudaFuncSetAttribute(mixed_jacobi_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shA);
             if (e != cudaSuccess) return e;
@@ -3118,7 +3115,13 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
                                                                                        (int)c0, nm, sc, flags);
             if ((e = cudaEventRecord(aux->jac_done[b], aux->s2)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(s, aux->jac_done[b], 0)) != cudaSuccess) return e;
-            kernB<<<(unsigned)nc, thB, shB, s>>>((float*)f, nx, ny, k, o, d_cut, beta, (int)c0, nm, sc, flags);
+            if (wide) {
+                const WideArgs wa{(float*)f, nx,      ny,        k,       o,      d_cut,  beta,   (int)c0, nm, sc.X,
+                                  mix_xr(nm), sc.lsq, sc.lidx, sc.pcount, sc.C32, sc.Clo, sc.C64, sc.b32,  sc.b64, flags};
+                if ((e = launch_analyze_wide(wa, nc, s)) != cudaSuccess) return e;
+            } else {
+                kernB<<<(unsigned)nc, 32, shB, s>>>((float*)f, nx, ny, k, o, d_cut, beta, (int)c0, nm, sc, flags);
+            }
             if ((e = cudaEventRecord(aux->ref_done[b], s)) != cudaSuccess) return e;
         }
     } else {
