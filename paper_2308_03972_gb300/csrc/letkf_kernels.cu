@@ -293,139 +293,6 @@ __device__ int jacobi_sym_warp(R* A, R* U, int n, int ld, int lane, R* rc, R* rs
     return -1;
 }
 
-// The cyclic Jacobi of jacobi_sym_warp (same rotations, same round-robin
-// order) for 33..128 (up to 64 pairs) by a block of NT = 256 threads: the
-// first 64 threads choose and apply the rotations of a round's pairs; then
-// every thread updates off-diagonal blocks and half a row of U (two threads
-// per row, 32 pairs each). The mask of rotated pairs alternates between two
-// shared slots by round parity, so it is not overwritten before every warp
-// has read it. mask: 4 words, red: NT / 32 floats. Binary32.
-template <int NT>
-__device__ int jacobi_sym_block(float* A, float* U, int n, int ld, float* rc, float* rs, int* rp, int* rq,
-                                unsigned* mask, float* red, float rel, int max_sweeps) {
-    static_assert(NT == 256, "two threads per row of U for n <= 128");
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    const int np = n + (n & 1);
-    const int half = np / 2;
-    const int nb = half * (half - 1) / 2;
-    float fro = 0.0f;
-    for (int e = tid; e < n * n; e += NT) {
-        const float v = A[(e / n) * ld + e % n];
-        fro += v * v;
-    }
-    fro = warp_sum(fro);
-    if (lane == 0) red[w] = fro;
-    __syncthreads();
-    fro = 0.0f;
-    for (int q = 0; q < NT / 32; ++q) fro += red[q];
-    const float thresh = rel * sqrtf(fro);
-    const int urow = tid >> 1, ut0 = (tid & 1) * 32;  // U: this thread's row and first pair
-    int parity = 0;
-    for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-        bool any_sweep = false;
-        for (int r = 0; r + 1 < np; ++r) {
-            unsigned* mk = mask + 2 * parity;
-            parity ^= 1;
-            if (w < 2) {
-                const int pr = tid;
-                bool rot = false;
-                if (pr < half) {
-                    const int pa = pr, pb = np - 1 - pr;
-                    const int P = pa == 0 ? 0 : 1 + (pa - 1 + r) % (np - 1);
-                    const int Q = 1 + (pb - 1 + r) % (np - 1);
-                    const int p = P < Q ? P : Q, q = P < Q ? Q : P;
-                    float c = 1.0f, sn = 0.0f;
-                    if (q < n) {
-                        const float apq = A[p * ld + q];
-                        if (fabsf(apq) > thresh) {
-                            const float app = A[p * ld + p], aqq = A[q * ld + q];
-                            const float th = aqq - app, ph = 2.0f * apq;
-                            const float rr = sqrtf(th * th + ph * ph);
-                            const float t = ph / (th >= 0.0f ? th + rr : th - rr);
-                            c = rsqrtf(1.0f + t * t);
-                            sn = t * c;
-                            rot = true;
-                            A[p * ld + p] = app - t * apq;
-                            A[q * ld + q] = aqq + t * apq;
-                            A[p * ld + q] = 0.0f;
-                            A[q * ld + p] = 0.0f;
-                        }
-                    }
-                    rp[pr] = p;
-                    rq[pr] = q;
-                    rc[pr] = c;
-                    rs[pr] = sn;
-                }
-                const unsigned bal = __ballot_sync(kFull, rot);
-                if (lane == 0) mk[w] = bal;
-            }
-            __syncthreads();
-            const unsigned long long any = mk[0] | ((unsigned long long)mk[1] << 32);
-            if (any == 0) continue;
-            any_sweep = true;
-            // Off-diagonal blocks (P, Q), P < Q: block bb is entry Q0 of row
-            // P of the pair matrix's upper triangle; a thread advances its
-            // previous (P, Q0) by NT blocks.
-            int P = 0, Q0 = 0;
-            for (int bb = tid; bb < nb; bb += NT) {
-                if (bb == tid) {
-                    Q0 = bb;
-                } else {
-                    Q0 += NT;
-                }
-                while (Q0 >= half - 1 - P) {
-                    Q0 -= half - 1 - P;
-                    ++P;
-                }
-                const int Q = P + 1 + Q0;
-                if (!((any >> P) & 1ull) && !((any >> Q) & 1ull)) continue;
-                const int pP = rp[P], qP = rq[P], pQ = rp[Q], qQ = rq[Q];
-                // The padding player of odd n (always a q) reads as zero and
-                // is not written.
-                const bool vP = qP < n, vQ = qQ < n;
-                const float cP = rc[P], sP = rs[P], cQ = rc[Q], sQ = rs[Q];
-                const float x00 = A[pP * ld + pQ];
-                const float x01 = vQ ? A[pP * ld + qQ] : 0.0f;
-                const float x10 = vP ? A[qP * ld + pQ] : 0.0f;
-                const float x11 = (vP && vQ) ? A[qP * ld + qQ] : 0.0f;
-                const float y00 = cP * x00 - sP * x10, y01 = cP * x01 - sP * x11;
-                const float y10 = sP * x00 + cP * x10, y11 = sP * x01 + cP * x11;
-                const float z00 = cQ * y00 - sQ * y01, z01 = sQ * y00 + cQ * y01;
-                const float z10 = cQ * y10 - sQ * y11, z11 = sQ * y10 + cQ * y11;
-                A[pP * ld + pQ] = z00;
-                A[pQ * ld + pP] = z00;
-                if (vQ) {
-                    A[pP * ld + qQ] = z01;
-                    A[qQ * ld + pP] = z01;
-                }
-                if (vP) {
-                    A[qP * ld + pQ] = z10;
-                    A[pQ * ld + qP] = z10;
-                }
-                if (vP && vQ) {
-                    A[qP * ld + qQ] = z11;
-                    A[qQ * ld + qP] = z11;
-                }
-            }
-            // U <- U J on this thread's half row.
-            if (urow < n) {
-                const int t1 = ut0 + 32 < half ? ut0 + 32 : half;
-                for (int t = ut0; t < t1; ++t) {
-                    if (!((any >> t) & 1ull)) continue;
-                    const int p = rp[t], q = rq[t];
-                    const float c = rc[t], sn = rs[t];
-                    const float up = U[urow * ld + p], uq = U[urow * ld + q];
-                    U[urow * ld + p] = c * up - sn * uq;
-                    U[urow * ld + q] = sn * up + c * uq;
-                }
-            }
-            __syncthreads();
-        }
-        if (!any_sweep) return sweep + 1;
-    }
-    return -1;
-}
-
 // Shared memory of the FP64 analysis kernel for problems up to NM.
 template <int NM>
 struct AnaSmem {
@@ -2238,30 +2105,78 @@ __global__ void __launch_bounds__(32 * kJacWarps, 4) mixed_jacobi_run_kernel(int
     }
 }
 
-// Kernel (A) for local problems of 33..128: the binary32 Jacobi of
-// jacobi_sym_block, kBlkThreads threads per grid point, same output.
-constexpr int kBlkThreads = 256;
-__host__ __device__ inline size_t jacobi_block_smem_bytes(int nm) {
-    return 2 * (size_t)nm * (nm + 1) * sizeof(float) + 64 * (2 * sizeof(float) + 2 * sizeof(int)) +
-           4 * sizeof(unsigned) + (kBlkThreads / 32) * sizeof(float) + sizeof(int);
+// Kernel (A) for local problems of 33..128: the cyclic Jacobi of
+// jacobi_sym_warp (same rotations, same round-robin order, stop at 1e-6
+// ||A||_F: the refinement of kernel (B) is second order in what remains) by a
+// block of WideShape<HM>::NT threads per grid point, HM the largest number of
+// pairs (32 or 64). The matrix is held by position in the tournament, not by
+// player: pair t of a round is always (top t, bottom t), and the round's
+// updates go out to where the next round has the players, a fixed permutation.
+//  * A (symmetric; entries of positions a < b only) in shared memory as four
+//    half x half quadrants (top/bottom row, top/bottom column): the 2 x 2
+//    block of pairs P < Q is four loads and four stores at addresses that a
+//    thread computes once, consecutive along Q. Two buffers, alternating.
+//  * U in the registers of threads of their own: a thread holds four pairs of
+//    kUR rows; players move on by register moves and two shuffles per row, so
+//    a round of U touches shared memory for the rotations only. Before, U
+//    went through shared memory (two thirds of the traffic that bound the
+//    kernel), and every access looked its pair up.
+// The entries see the rotations in the same order with the same roundings as
+// before; the result is the same to the bit.
+constexpr int kUR = 4;            // rows of U per thread
+constexpr int kBlkThreads = 256;  // threads that load the matrix
+
+template <int HM>
+struct WideShape {
+    static constexpr int LPR = HM / 4;                    // threads per row of U
+    static constexpr int NA = HM == 32 ? 128 : 256;       // threads that update A
+    static constexpr int NU = 2 * HM / kUR * LPR;         // threads that hold U: 128 or 512
+    static constexpr int NT = NA + NU;
+    static constexpr int LD = HM + 1;
+    static constexpr int QUAD = HM * LD;                  // floats per quadrant
+    static constexpr int BUF = 4 * QUAD + 2 * HM;         // quadrants and diagonal
+    static constexpr int NB = (HM * (HM - 1) / 2 + NA - 1) / NA;  // blocks per thread
+    static constexpr size_t bytes() { return (2 * BUF + 2 * 2 * 4 * HM + 16) * sizeof(float); }
+};
+
+// Position of player i before the first round of a sweep: pair (times two), plus one at the bottom.
+__device__ __forceinline__ int wide_slot(int i, int np) { return i < np / 2 ? 2 * i : 2 * (np - 1 - i) + 1; }
+// Where the player of a position is in the next round.
+__device__ __forceinline__ int wide_next(int s, int half) {
+    if (s == 0 || half == 1) return s;
+    if (s == 2) return 1;
+    if (s == 2 * half - 1) return 2 * half - 2;
+    return (s & 1) ? s + 2 : s - 2;
+}
+// Address of entry (a, b) of the symmetric matrix, positions a != b.
+template <int HM>
+__device__ __forceinline__ int wide_at(int a, int b) {
+    const int lo = a < b ? a : b, hi = a < b ? b : a;
+    return ((lo & 1) * 2 + (hi & 1)) * WideShape<HM>::QUAD + (lo >> 1) * WideShape<HM>::LD + (hi >> 1);
+}
+// The rotation of a pair's values, u at the top. With p the lower player's
+// value and q the other's, p' = fma(c, p, -(s q)) and q' = fma(s, p, c q);
+// flip says that the top holds q, and the coefficients (x, y for the top, z,
+// w for the bottom) come sorted accordingly.
+__device__ __forceinline__ void wide_rot(const float4& k, bool flip, float& u, float& v) {
+    const float p = flip ? v : u, q = flip ? u : v;
+    u = __fmaf_rn(k.x, p, __fmul_rn(k.y, q));
+    v = __fmaf_rn(k.z, p, __fmul_rn(k.w, q));
 }
 
-__global__ void __launch_bounds__(kBlkThreads, 5) mixed_jacobi_block_kernel(int nx, int ny, int k, ObsParams o,
-                                                                         double d_cut, double beta,
-                                                                         int cell0, int nm, MixScratch sc,
-                                                                         int* __restrict__ flags) {
+template <int HM>
+__global__ void __launch_bounds__(WideShape<HM>::NT, HM == 32 ? 4 : 1) mixed_jacobi_wide_kernel(
+    int nx, int ny, int k, ObsParams o, double d_cut, double beta, int cell0, int nm, MixScratch sc,
+    int* __restrict__ flags) {
+    using WS = WideShape<HM>;
+    constexpr int NA = WS::NA, LD = WS::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    float* buf = reinterpret_cast<float*>(smem_raw);                // two buffers
+    // Rotations by round parity: [2][HM] by pair, then [2][4][HM / 4] as U's threads read them.
+    float4* cs = reinterpret_cast<float4*>(buf + 2 * WS::BUF);
+    float* red = reinterpret_cast<float*>(cs + 4 * HM);             // [8], then p
+    int* pshare = reinterpret_cast<int*>(red + 8);
     const int nobs = o.nvar * o.npts;
-    const int ld = nm + 1;
-    float* A = reinterpret_cast<float*>(smem_raw);
-    float* U = A + (size_t)nm * ld;
-    float* rc = U + (size_t)nm * ld;
-    float* rs = rc + 64;
-    int* rp = reinterpret_cast<int*>(rs + 64);
-    int* rq = rp + 64;
-    unsigned* mask = reinterpret_cast<unsigned*>(rq + 64);
-    float* red = reinterpret_cast<float*>(mask + 4);
-    int* pshare = reinterpret_cast<int*>(red + kBlkThreads / 32);
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int li = blockIdx.x;
     const int cell = cell0 + li;
@@ -2276,44 +2191,221 @@ __global__ void __launch_bounds__(kBlkThreads, 5) mixed_jacobi_block_kernel(int 
             *pshare = p;
         }
     }
+    for (int e = tid; e < 2 * WS::BUF; e += WS::NT) buf[e] = 0.0f;
     __syncthreads();
     const int p = *pshare;
     if (p == 0 || p > cap) return;  // p > cap: reported by kernel (B)
     const bool obs_space = p < k;
     const int n = obs_space ? p : k;
     if (n > nm) return;  // reported by kernel (B)
+    const int np = n + (n & 1), half = np / 2;
     const double aa = (k - 1) / beta;
-    for (int e = tid; e < n * n; e += kBlkThreads) {
-        const int i = e / n, c = e % n;
-        float v;
-        if (obs_space) {
-            v = (float)(lsq[i] * o.G[(size_t)lidx[i] * nobs + lidx[c]] * lsq[c]);
-        } else if (sc.C32) {
-            v = sc.C32[(size_t)li * k * k + (size_t)i * k + c];
-        } else if (sc.C64) {
-            v = (float)sc.C64[(size_t)li * k * k + (size_t)i * k + c];
-        } else {
-            double s = (i == c) ? aa : 0.0;
-            for (int l = 0; l < p; ++l) {
-                const double* row = o.dY + (size_t)lidx[l] * k;
-                s += lsq[l] * lsq[l] * row[i] * row[c];
+    float fro = 0.0f;
+    if (tid < kBlkThreads) {
+        for (int e = tid; e < n * n; e += kBlkThreads) {
+            const int i = e / n, c = e % n;
+            float v;
+            if (obs_space) {
+                v = (float)(lsq[i] * o.G[(size_t)lidx[i] * nobs + lidx[c]] * lsq[c]);
+            } else if (sc.C32) {
+                v = sc.C32[(size_t)li * k * k + (size_t)i * k + c];
+            } else if (sc.C64) {
+                v = (float)sc.C64[(size_t)li * k * k + (size_t)i * k + c];
+            } else {
+                double s = (i == c) ? aa : 0.0;
+                for (int l = 0; l < p; ++l) {
+                    const double* row = o.dY + (size_t)lidx[l] * k;
+                    s += lsq[l] * lsq[l] * row[i] * row[c];
+                }
+                v = (float)s;
             }
-            v = (float)s;
+            const int si = wide_slot(i, np);
+            if (i == c)
+                buf[4 * WS::QUAD + si] = v;
+            else if (si < wide_slot(c, np))
+                buf[wide_at<HM>(si, wide_slot(c, np))] = v;
+            fro += v * v;
         }
-        A[i * ld + c] = v;
-        U[i * ld + c] = (i == c) ? 1.0f : 0.0f;
+        fro = warp_sum(fro);
+        if (lane == 0) red[w] = fro;
     }
     __syncthreads();
-    // Stop at 1e-6 ||A||_F: the refinement of kernel (B) is second order in
-    // what remains.
-    const int sweeps = jacobi_sym_block<kBlkThreads>(A, U, n, ld, rc, rs, rp, rq, mask, red, 1e-6f, kMaxSweeps);
+    fro = 0.0f;
+    for (int q = 0; q < kBlkThreads / 32; ++q) fro += red[q];
+    const float thresh = 1e-6f * sqrtf(fro);
+
+    // Roles: threads below NA update A (the first half of them also rotate a
+    // pair each), the others hold U.
+    const bool on_a = tid < NA;
+    const int nb = half * (half - 1) / 2;
+    int pq[WS::NB];                     // P, Q of this thread's blocks
+    unsigned to0[WS::NB], to1[WS::NB];  // where their entries go, two 16-bit addresses each
+    int d0 = 0, d1 = 0, dto = 0;        // where the pair's diagonal and off-diagonal entries go
+    if (on_a) {
+        int P = 0, Q0 = tid;
+#pragma unroll
+        for (int i = 0; i < WS::NB; ++i) {
+            pq[i] = -1;
+            to0[i] = to1[i] = 0;
+            if (tid + i * NA < nb) {
+                while (Q0 >= half - 1 - P) {
+                    Q0 -= half - 1 - P;
+                    ++P;
+                }
+                const int Q = P + 1 + Q0;
+                pq[i] = P | (Q << 8);
+                const int a0 = wide_next(2 * P, half), a1 = wide_next(2 * P + 1, half);
+                const int b0 = wide_next(2 * Q, half), b1 = wide_next(2 * Q + 1, half);
+                to0[i] = (unsigned)wide_at<HM>(a0, b0) | ((unsigned)wide_at<HM>(a0, b1) << 16);
+                to1[i] = (unsigned)wide_at<HM>(a1, b0) | ((unsigned)wide_at<HM>(a1, b1) << 16);
+                Q0 += NA;
+            }
+        }
+        if (tid < half) {
+            d0 = wide_next(2 * tid, half);
+            d1 = wide_next(2 * tid + 1, half);
+            dto = wide_at<HM>(d0, d1);
+        }
+    }
+    const int ul = (tid - NA) % WS::LPR, us = (tid - NA) / WS::LPR;  // U: place in the row, first row
+    const int ulast = half - 1 - 4 * ul;                            // which of the four pairs is the last one
+    constexpr int URS = 2 * HM / kUR;                               // U: stride of the rows
+    float ut[kUR][4], ub[kUR][4];
+#pragma unroll
+    for (int r = 0; r < kUR; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int t = 4 * ul + q, row = us + URS * r;
+            ut[r][q] = t < half && row == t ? 1.0f : 0.0f;
+            ub[r][q] = t < half && row == np - 1 - t ? 1.0f : 0.0f;
+        }
+
+    int cur = 0, sweeps = -1;
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+        // A sweep that would rotate nothing is found in one pass.
+        bool big = false;
+        if (on_a) {
+            const float* A = buf + cur * WS::BUF;
+#pragma unroll
+            for (int i = 0; i < WS::NB; ++i)
+                if (pq[i] >= 0) {
+                    const float* a = A + (pq[i] & 255) * LD + (pq[i] >> 8);
+                    big |= fabsf(a[0]) > thresh || fabsf(a[WS::QUAD]) > thresh || fabsf(a[2 * WS::QUAD]) > thresh ||
+                           fabsf(a[3 * WS::QUAD]) > thresh;
+                }
+            if (tid < half) big |= fabsf(A[WS::QUAD + tid * (LD + 1)]) > thresh;
+        }
+        if (!__syncthreads_or(big)) {
+            sweeps = sweep + 1;
+            break;
+        }
+        for (int r = 0; r + 1 < np; ++r) {
+            const float* A = buf + cur * WS::BUF;
+            float* B = buf + (cur ^ 1) * WS::BUF;
+            float4* rot = cs + cur * HM;
+            // Pairs 1 .. flips hold the lower player at the bottom.
+            const int flips = r < np - r ? r - 1 : np - 1 - r;
+            if (tid < half) {
+                const float at = A[4 * WS::QUAD + 2 * tid], ab = A[4 * WS::QUAD + 2 * tid + 1];
+                float apq = A[WS::QUAD + tid * (LD + 1)];
+                const bool flip = tid > 0 && tid <= flips;
+                float app = flip ? ab : at, aqq = flip ? at : ab;
+                float c = 1.0f, sn = 0.0f;
+                if (fabsf(apq) > thresh) {
+                    const float th = aqq - app, ph = 2.0f * apq;
+                    const float rr = sqrtf(__fmaf_rn(ph, ph, __fmul_rn(th, th)));
+                    const float t = ph / (th >= 0.0f ? th + rr : th - rr);
+                    c = rsqrtf(1.0f + t * t);
+                    sn = t * c;
+                    app = app - t * apq;
+                    aqq = aqq + t * apq;
+                    apq = 0.0f;
+                }
+                const float4 rk = flip ? make_float4(sn, c, c, -sn) : make_float4(c, -sn, sn, c);
+                rot[tid] = rk;
+                rot[2 * HM + (tid & 3) * (HM / 4) + (tid >> 2)] = rk;
+                B[4 * WS::QUAD + d0] = flip ? aqq : app;
+                B[4 * WS::QUAD + d1] = flip ? app : aqq;
+                B[dto] = apq;
+            }
+            __syncthreads();
+            if (on_a) {
+#pragma unroll
+                for (int i = 0; i < WS::NB; ++i) {
+                    if (pq[i] < 0) continue;
+                    const int P = pq[i] & 255, Q = pq[i] >> 8;
+                    const float4 rp = rot[P], rq = rot[Q];
+                    const bool fp = P > 0 && P <= flips, fq = Q <= flips;
+                    const float* a = A + P * LD + Q;
+                    float x00 = a[0], x01 = a[WS::QUAD], x10 = a[2 * WS::QUAD], x11 = a[3 * WS::QUAD];
+                    wide_rot(rp, fp, x00, x10);
+                    wide_rot(rp, fp, x01, x11);
+                    wide_rot(rq, fq, x00, x01);
+                    wide_rot(rq, fq, x10, x11);
+                    B[to0[i] & 0xffffu] = x00;
+                    B[to0[i] >> 16] = x01;
+                    B[to1[i] & 0xffffu] = x10;
+                    B[to1[i] >> 16] = x11;
+                }
+                // The next round's pairs read what these threads wrote; the
+                // threads of U meet them at the next round's barrier.
+                asm volatile("bar.sync 1, %0;" ::"n"(NA) : "memory");
+            } else {
+                float4 rc[4];
+                bool rf[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    rc[q] = rot[2 * HM + q * (HM / 4) + ul];
+                    rf[q] = 4 * ul + q > 0 && 4 * ul + q <= flips;
+                }
+#pragma unroll
+                for (int j = 0; j < kUR; ++j) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) wide_rot(rc[q], rf[q], ut[j][q], ub[j][q]);
+                    // Tops move down a pair, bottoms up; the last top and the
+                    // first bottom change sides, the first top stays.
+                    const float tn = __shfl_down_sync(kFull, ut[j][0], 1, WS::LPR);
+                    const float bp = __shfl_up_sync(kFull, ub[j][3], 1, WS::LPR);
+                    float nt[4], nbt[4];
+                    nt[0] = ul == 0 ? ut[j][0] : ut[j][1];
+                    nt[1] = ut[j][2];
+                    nt[2] = ut[j][3];
+                    nt[3] = tn;
+                    nbt[0] = ul == 0 ? ut[j][1] : bp;
+                    nbt[1] = ub[j][0];
+                    nbt[2] = ub[j][1];
+                    nbt[3] = ub[j][2];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (q == ulast) nt[q] = ub[j][q];
+                    if (half > 1)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            ut[j][q] = nt[q];
+                            ub[j][q] = nbt[q];
+                        }
+                }
+            }
+            cur ^= 1;
+        }
+    }
     if (sweeps < 0 && tid == 0) atomicOr(flags, FLAG_NOCONV);
     if (w == 0) record_sweeps(o, sweeps, lane);
-    const int xr = mix_xr(nm);
-    float* Xp = sc.X + (size_t)li * xr * xr;
-    for (int e = tid; e < n * n; e += kBlkThreads) {
-        const int i = e / n, c = e % n;
-        Xp[(size_t)i * xr + c] = U[i * ld + c];
+    if (!on_a) {
+        const int xr = mix_xr(nm);
+        float* Xp = sc.X + (size_t)li * xr * xr;
+#pragma unroll
+        for (int j = 0; j < kUR; ++j) {
+            const int row = us + URS * j;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int t = 4 * ul + q;
+                if (row < n && t < half) {
+                    Xp[(size_t)row * xr + t] = ut[j][q];
+                    if (np - 1 - t < n) Xp[(size_t)row * xr + np - 1 - t] = ub[j][q];
+                }
+            }
+        }
     }
 }
 
@@ -3049,14 +3141,17 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         const int cap = o.plmax > 0 ? o.plmax : nobs;
         const size_t shB = mix_smem_bytes(k, cap, nm);
         const bool wide = nm > NREG;
-        const size_t shA = wide ? jacobi_block_smem_bytes(nm) : 0;
+        const bool big = nm > NMID;
+        const auto kernA = big ? mixed_jacobi_wide_kernel<64> : mixed_jacobi_wide_kernel<32>;
+        const size_t shA = big ? WideShape<64>::bytes() : WideShape<32>::bytes();
+        const int thA = big ? WideShape<64>::NT : WideShape<32>::NT;
         const auto kernB = analyze_mixed_kernel<false, false, 1>;
         if (!wide) {
             e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
             if (e != cudaSuccess) return e;
         }
         if (wide) {
-            e = cudaFuncSetAttribute(mixed_jacobi_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shA);
+            e = cudaFuncSetAttribute(kernA, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shA);
             if (e != cudaSuccess) return e;
         }
         const int kg = gram_k(fp32, k, prod), gsz = gram_sz(prod);
@@ -3111,8 +3206,7 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
                 mixed_jacobi_kernel<<<(unsigned)((nc + kJacWarps - 1) / kJacWarps), 32 * kJacWarps, 0,
                                       aux->s2>>>(nx, ny, k, o, d_cut, beta, (int)c0, nc, nm, sc, flags);
             else
-                mixed_jacobi_block_kernel<<<(unsigned)nc, kBlkThreads, shA, aux->s2>>>(nx, ny, k, o, d_cut, beta,
-                                                                                       (int)c0, nm, sc, flags);
+                kernA<<<(unsigned)nc, thA, shA, aux->s2>>>(nx, ny, k, o, d_cut, beta, (int)c0, nm, sc, flags);
             if ((e = cudaEventRecord(aux->jac_done[b], aux->s2)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(s, aux->jac_done[b], 0)) != cudaSuccess) return e;
             if (wide) {
