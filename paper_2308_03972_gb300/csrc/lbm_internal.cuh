@@ -176,7 +176,7 @@ cudaError_t launch_gram_outer(const GramArgs& g, double aa, cudaStream_t s);
 
 // ---- letkf_wide.cu --------------------------------------------------------
 // Refinement and update (kernel (B)) of the grid points cell0 .. of a chunk
-// with local problems up to nm, 32 < nm <= 128, from kernel (A)'s basis X
+// with local problems up to nm, 16 < nm <= 128, from kernel (A)'s basis X
 // [.][xr][xr], local lists lsq, lidx and counts pcount, and the Gram pass's C
 // (C32 with or without Clo, or C64) and b (b32 or b64).
 struct WideArgs {

@@ -9,7 +9,7 @@
 // (outer_kernel); the pass over the grid points is then one product of the
 // weights with them: per grid point k (k + 1) / 2 entries times the local
 // points, against k^2 entries times nvar as many scalars when the rows
-// themselves are multiplied (up to 32 members; launch_analyze says why).
+// themselves are multiplied (up to 32 members; gram_by_outer says why).
 //
 // gram_outer_kernel is bound by the binary32 pipe (twelve operations per
 // multiply-add: the exact product, the two cross terms, TwoSum and the error

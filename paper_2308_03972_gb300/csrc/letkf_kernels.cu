@@ -36,7 +36,7 @@ namespace lbmgpu {
 namespace {
 
 constexpr int NMAX = 128;  // largest local eigenproblem of the mixed-precision analysis
-constexpr int NMID = 64;   // largest held wholly in shared memory; the FP64 analysis' limit
+constexpr int NMID = 64;   // largest of the smaller wide shapes; the FP64 analysis' limit
 constexpr int NREG = 32;   // largest one handled by the register Jacobi
 constexpr int kMaxSweeps = 30;
 
@@ -150,25 +150,10 @@ __device__ int local_set(const ObsParams& o, int x, int y, int nx, int ny, doubl
 }
 
 // ------------------------------------------------------------------ K3, FP64
-// Apply body(c) to the columns c a thread owns: c = lane when every problem
-// fits one lane per column (WIDE = false), else c = t, t + 32 NW, ... for
-// thread t of NW warps.
-template <bool WIDE, int NW = 1, typename F>
-__device__ __forceinline__ void for_cols(int t, int n, F&& body) {
-    if (WIDE) {
-        for (int c = t; c < n; c += 32 * NW) body(c);
-    } else if (t < n) {
-        body(t);
-    }
-}
-
-// Barrier of the NW warps that share a grid point.
-template <int NW>
-__device__ __forceinline__ void point_sync() {
-    if (NW == 1)
-        __syncwarp();
-    else
-        __syncthreads();
+// Apply body to the lane's column.
+template <typename F>
+__device__ __forceinline__ void for_col(int t, int n, F&& body) {
+    if (t < n) body(t);
 }
 
 __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
@@ -1223,7 +1208,6 @@ struct MixScratch {
     int* pcount;   // [chunk] number of local scalars
     float* C32;    // [chunk][k][k] a I + Yh^T Yh from the reduced-precision Gram, or null
     float* b32;    // [chunk][k] Yh^T d-hat from the same pass, or null
-    float* big;    // [chunk][4][nm][ld] kernel (B)'s A and A Y halves when nm > NMID, or null
     double* C64;   // [chunk][k][k] a I + Yh^T Yh from the FP64 Gram pass, or null
     double* b64;   // [chunk][k] Yh^T d-hat from the same pass, or null
     // Double-binary32 Gram pass: C as two binary32 planes in C64's space,
@@ -1248,18 +1232,12 @@ __host__ __device__ inline int mix_xr(int nm) { return nm <= NREG ? NREG : (nm <
 // Row stride of the matrices of kernel (B): nm + 1 rounded to odd.
 __host__ __device__ inline int mix_ld(int nm) { return (nm % 2 == 0) ? nm + 1 : nm; }
 
-// Floats per grid point of kernel (B)'s matrices kept in global scratch
-// (A and A Y, two binary32 halves each) when nm > NMID, else 0.
-__host__ __device__ inline size_t mix_big_floats(int nm) {
-    return nm > NMID ? 4 * (size_t)nm * mix_ld(nm) : 0;
-}
-
 // kg: members k when a Gram pass is used (its C and b per point), else 0;
 // gsz: bytes of its elements (4 reduced precision, 8 FP64).
 __host__ __device__ inline size_t mix_scratch_bytes_per_point(int nobs, int nm, int kg, int gsz) {
     const int xr = mix_xr(nm);
     return (size_t)xr * xr * sizeof(float) + (size_t)nobs * (sizeof(double) + sizeof(int)) +
-           sizeof(int) + (size_t)kg * (kg + 1) * gsz + mix_big_floats(nm) * sizeof(float);
+           sizeof(int) + (size_t)kg * (kg + 1) * gsz;
 }
 
 // Grid points per chunk: up to kChunkCells, with at most 384 MiB of scratch
@@ -1295,8 +1273,6 @@ __host__ __device__ inline MixScratch mix_scratch_at(void* base, long long chunk
     m.b32 = (kg && gsz == 4) ? reinterpret_cast<float*>(p) : nullptr;
     m.b64 = (kg && gsz == 8) ? reinterpret_cast<double*>(p) : nullptr;
     m.Clo = nullptr;
-    p += (size_t)chunk * kg * gsz;
-    m.big = nm > NMID ? reinterpret_cast<float*>(p) : nullptr;
     return m;
 }
 
@@ -1897,6 +1873,27 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_df_kernel(int nx,
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int li0 = blockIdx.x * kGramPts;
     const int nv = o.nvar;
+    if (K <= kOuterMaxK) {
+        // After the outer-product pass: only blocks where some entry's low
+        // half lies within 2^-44 of the largest diagonal entry of half a unit
+        // in the last place of the high half (half of that just above a power
+        // of two).
+        bool near = false;
+        if (li0 + w < ncell) {
+            const float* Ch = sc.C32 + (size_t)(li0 + w) * k * k;
+            const float* Cl = sc.Clo + (size_t)(li0 + w) * k * k;
+            float dm = lane < k ? Ch[lane * k + lane] : 0.0f;
+#pragma unroll
+            for (int t = 16; t > 0; t >>= 1) dm = fmaxf(dm, __shfl_xor_sync(kFull, dm, t));
+            const float tau = 5.7e-14f * dm;
+            for (int e = lane; e < k * k; e += 32) {
+                const unsigned b = __float_as_uint(Ch[e]) & 0x7fffffffu;
+                const float half = b >= (25u << 23) ? __uint_as_float((b & 0x7f800000u) - (24u << 23)) : 0.0f;
+                near |= fabsf(fabsf(Cl[e]) - half) <= tau || ((b & 0x7fffffu) == 0u && b != 0u);
+            }
+        }
+        if (!__syncthreads_or(near)) return;
+    }
     const int total = gram_merge(o, nx, ny, d_cut, cell0, li0, ncell, U, pcnt, wcount);
     const long long lim2 = support_lim2(d_cut);
     const float aah = (float)aa, aal = (float)(aa - (double)aah);  // a = aah + aal
@@ -2267,15 +2264,15 @@ __global__ void __launch_bounds__(WideShape<HM>::NT, HM == 32 ? 4 : 1) mixed_jac
             dto = wide_at<HM>(d0, d1);
         }
     }
-    const int ul = (tid - NA) % WS::LPR, us = (tid - NA) / WS::LPR;  // U: place in the row, first row
+    const int ul = (tid - NA) % WS::LPR, us = (tid - NA) / WS::LPR;  // U: place in the row, rows kUR us ..
     const int ulast = half - 1 - 4 * ul;                            // which of the four pairs is the last one
-    constexpr int URS = 2 * HM / kUR;                               // U: stride of the rows
+    const bool u_on = (tid - NA) / 32 * 32 / WS::LPR * kUR < n;     // some row of this warp exists
     float ut[kUR][4], ub[kUR][4];
 #pragma unroll
     for (int r = 0; r < kUR; ++r)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int t = 4 * ul + q, row = us + URS * r;
+            const int t = 4 * ul + q, row = kUR * us + r;
             ut[r][q] = t < half && row == t ? 1.0f : 0.0f;
             ub[r][q] = t < half && row == np - 1 - t ? 1.0f : 0.0f;
         }
@@ -2350,7 +2347,7 @@ __global__ void __launch_bounds__(WideShape<HM>::NT, HM == 32 ? 4 : 1) mixed_jac
                 // The next round's pairs read what these threads wrote; the
                 // threads of U meet them at the next round's barrier.
                 asm volatile("bar.sync 1, %0;" ::"n"(NA) : "memory");
-            } else {
+            } else if (u_on) {
                 float4 rc[4];
                 bool rf[4];
 #pragma unroll
@@ -2396,7 +2393,7 @@ __global__ void __launch_bounds__(WideShape<HM>::NT, HM == 32 ? 4 : 1) mixed_jac
         float* Xp = sc.X + (size_t)li * xr * xr;
 #pragma unroll
         for (int j = 0; j < kUR; ++j) {
-            const int row = us + URS * j;
+            const int row = kUR * us + j;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int t = 4 * ul + q;
@@ -2419,8 +2416,8 @@ struct MixSmem {
     float* Wh;     // [nm][ld] A Y, high half; then f(S) in binary32 (F32), then T
     float* Wl;     // [nm][ld] A Y, low half
     float* Y32;    // [nm][ld] the basis (binary32, exact)
-    float* E32;    // [nm][ld] E = Y^T Y - I (non-orthogonality of the basis); up to
-                   // NMID it shares Al's space (A's low half is dead once A Y is formed)
+    float* E32;    // [nm][ld] E = Y^T Y - I (non-orthogonality of the basis), in Al's
+                   // space (A's low half is dead once A Y is formed)
     double* lsq;   // [nl]
     double* ldh;   // [nl]
     double* vb;    // [nm]
@@ -2438,20 +2435,17 @@ struct MixSmem {
     int* lidx;     // [nl]
 };
 
-// Up to NMID five matrices (E32 shares Al's space): at n = 28 and k = 64,
-// 22.3 KB per grid point, ten points per SM. Above NMID, Ah, Al, Wh and Wl
-// live in the global scratch (MixScratch::big) and shared memory holds Y32
-// and E32.
+// Five matrices (E32 shares Al's space): at n = 28 and k = 64, 22.3 KB per
+// grid point, ten points per SM.
 __host__ __device__ inline size_t mix_smem_bytes(int k, int nl, int nm) {
     const int ld = mix_ld(nm);
     const size_t d = 2 * (size_t)nl + 2 * (size_t)nm;
-    const size_t f = (nm > NMID ? 2 : 5) * (size_t)nm * ld + 9 * (size_t)k + 16 + 18 * (size_t)nm + 16 +
+    const size_t f = 5 * (size_t)nm * ld + 9 * (size_t)k + 16 + 18 * (size_t)nm + 16 +
                      5 * (size_t)nm;
     return d * sizeof(double) + ((f * sizeof(float) + 7) / 8) * 8 + (size_t)nl * sizeof(int);
 }
 
-// big: this grid point's 4 nm ld floats of global scratch, or null.
-__device__ inline MixSmem carve_mix(unsigned char* raw, int k, int nl, int nm, float* big) {
+__device__ inline MixSmem carve_mix(unsigned char* raw, int k, int nl, int nm) {
     const int ld = mix_ld(nm);
     MixSmem s;
     double* p = reinterpret_cast<double*>(raw);
@@ -2464,24 +2458,17 @@ __device__ inline MixSmem carve_mix(unsigned char* raw, int k, int nl, int nm, f
     s.dS = p;
     p += nm;
     float* q = reinterpret_cast<float*>(p);
-    float* m = big ? big : q;
-    s.Ah = m;
-    m += nm * ld;
-    s.Al = m;
-    m += nm * ld;
-    s.Wh = m;
-    m += nm * ld;
-    s.Wl = m;
-    m += nm * ld;
-    if (!big) q = m;
+    s.Ah = q;
+    q += nm * ld;
+    s.Al = q;
+    q += nm * ld;
+    s.Wh = q;
+    q += nm * ld;
+    s.Wl = q;
+    q += nm * ld;
     s.Y32 = q;
     q += nm * ld;
-    if (big) {
-        s.E32 = q;
-        q += nm * ld;
-    } else {
-        s.E32 = s.Al;
-    }
+    s.E32 = s.Al;
     s.dX = q;
     q += 9 * k;
     s.xbar = q;
@@ -2511,12 +2498,12 @@ __device__ inline MixSmem carve_mix(unsigned char* raw, int k, int nl, int nm, f
 
 // C = P^T Q over the upper triangle (mirrored) in double-binary32: P binary32,
 // Q = Qhi + Qlo (Qlo may be null). store(i, j, value) writes both halves.
-// Thread t of NW warps takes entries t, t + 32 NW, ...
-template <int NW = 1, typename Store>
+// Lane t takes entries t, t + 32, ...
+template <typename Store>
 __device__ void sym_product_df(const float* P, const float* Qhi, const float* Qlo, int n, int ld, int t,
                                Store&& store) {
     const int ne = n * (n + 1) / 2;
-    for (int e0 = t; e0 < ne; e0 += 32 * NW) {
+    for (int e0 = t; e0 < ne; e0 += 32) {
         int i = 0, j = e0;
         while (j >= n - i) {
             j -= n - i;
@@ -2544,11 +2531,10 @@ __device__ void sym_product_df(const float* P, const float* Qhi, const float* Ql
 // diagonal of S' in dS (FP64) and its off-diagonal in Soff (binary32: the
 // entries are ~1e-6 of |A| and enter the matrix functions to first order).
 // Soff may alias Ah and E32 may alias Al (A is not read after A Y).
-template <bool WIDE, int NW = 1>
 __device__ void refine_rr(const float* Ah, const float* Al, const float* Y32, float* Wh, float* Wl,
                           float* E32, float* Soff, double* dS, int n, int ld, int t) {
     // W = A Y, column col: four rows at a time, then the remainder.
-    for_cols<WIDE, NW>(t, n, [&](int col) {
+    for_col(t, n, [&](int col) {
         int i0 = 0;
         for (; i0 + 3 < n; i0 += 4) {
             float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -2567,15 +2553,15 @@ __device__ void refine_rr(const float* Ah, const float* Al, const float* Y32, fl
             two_sum(s, c, Wh[i0 * ld + col], Wl[i0 * ld + col]);
         }
     });
-    point_sync<NW>();
+    __syncwarp();
     // E = Y^T Y - I.
-    sym_product_df<NW>(Y32, Y32, nullptr, n, ld, t, [&](int i, int j, double v) {
+    sym_product_df(Y32, Y32, nullptr, n, ld, t, [&](int i, int j, double v) {
         const float e = (float)(v - (i == j ? 1.0 : 0.0));
         E32[i * ld + j] = e;
         E32[j * ld + i] = e;
     });
     // S = Y^T (A Y), symmetric: diagonal to dS, off-diagonal to Soff.
-    sym_product_df<NW>(Y32, Wh, Wl, n, ld, t, [&](int i, int j, double v) {
+    sym_product_df(Y32, Wh, Wl, n, ld, t, [&](int i, int j, double v) {
         if (i == j) {
             dS[i] = v;
         } else {
@@ -2583,24 +2569,22 @@ __device__ void refine_rr(const float* Ah, const float* Al, const float* Y32, fl
             Soff[j * ld + i] = (float)v;
         }
     });
-    point_sync<NW>();
+    __syncwarp();
     // S' = S - E o (d_i + d_j)/2 (the diagonal last, after every thread has
     // read the uncorrected one).
-    for_cols<WIDE, NW>(t, n, [&](int c) {
+    for_col(t, n, [&](int c) {
         const double dc = dS[c];
         for (int i = 0; i < n; ++i)
             if (i != c)
                 Soff[i * ld + c] = (float)((double)Soff[i * ld + c] - (double)E32[i * ld + c] * 0.5 * (dS[i] + dc));
     });
-    point_sync<NW>();
-    for_cols<WIDE, NW>(t, n, [&](int c) { dS[c] -= (double)E32[c * ld + c] * dS[c]; });
-    point_sync<NW>();
+    __syncwarp();
+    for_col(t, n, [&](int c) { dS[c] -= (double)E32[c * ld + c] * dS[c]; });
+    __syncwarp();
 }
 
-// BIG (nm > NMID): A and A Y in global scratch (L2-resident), the rest as
-// below. NW warps share a grid point (1 up to NREG).
-template <bool WIDE, bool BIG, int NW>
-__global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restrict__ f, int nx, int ny,
+// Kernel (B) for local problems up to 16 (launch_analyze), one warp per grid point.
+__global__ void __launch_bounds__(32) analyze_mixed_kernel(float* __restrict__ f, int nx, int ny,
                                                            int k, ObsParams o, double d_cut,
                                                            double beta, int cell0, int nm,
                                                            MixScratch sc,
@@ -2609,16 +2593,15 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
     const int nobs = o.nvar * o.npts;
     const int cap = o.plmax > 0 ? o.plmax : nobs;
     const int li = blockIdx.x;
-    MixSmem sm = carve_mix(smem_raw, k, cap, nm, BIG ? sc.big + (size_t)li * mix_big_floats(nm) : nullptr);
+    MixSmem sm = carve_mix(smem_raw, k, cap, nm);
     const int ld = mix_ld(nm);
-    constexpr int NTH = 32 * NW;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int lane = threadIdx.x;
     const int cell = cell0 + li;
     const size_t plane = (size_t)nx * ny * k;
     float* fc = f + (size_t)cell * k;
 
     // Ensemble mean and perturbations in binary32.
-    for (int a = wid; a < 9; a += NW) {  // one warp per component
+    for (int a = 0; a < 9; ++a) {
         float s = 0.0f;
         for (int m = lane; m < k; m += 32) {
             const float xv = fc[a * plane + m];
@@ -2633,28 +2616,28 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
     // Local set from kernel (A).
     const int p = sc.pcount[li];
     if (p > cap) {
-        if (tid == 0) atomicOr(flags, FLAG_TOOLARGE);
+        if (lane == 0) atomicOr(flags, FLAG_TOOLARGE);
         return;
     }
-    for (int i = tid; i < p; i += NTH) {
+    for (int i = lane; i < p; i += 32) {
         const int oi = sc.lidx[(size_t)li * cap + i];
         const double si = sc.lsq[(size_t)li * cap + i];
         sm.lidx[i] = oi;
         sm.lsq[i] = si;
         sm.ldh[i] = si * o.d[oi];
     }
-    point_sync<NW>();
+    __syncwarp();
 
     if (p == 0) {
         const float sb = (float)sqrt(beta);
         for (int a = 0; a < 9; ++a)
-            for (int m = tid; m < k; m += NTH) fc[a * plane + m] = sm.xbar[a] + sb * sm.dX[a * k + m];
+            for (int m = lane; m < k; m += 32) fc[a * plane + m] = sm.xbar[a] + sb * sm.dX[a * k + m];
         return;
     }
     const bool obs_space = p < k;
     const int n = obs_space ? p : k;
     if (n > nm) {
-        if (tid == 0) atomicOr(flags, FLAG_TOOLARGE);
+        if (lane == 0) atomicOr(flags, FLAG_TOOLARGE);
         return;
     }
     const double aa = (k - 1) / beta;
@@ -2668,9 +2651,9 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
     // The symmetric matrix in FP64: A = Yh Yh^T (observation space) or
     // C = a I + Yh^T Yh with b = Yh^T d-hat (ensemble space); the basis X
     // from kernel (A).
-    const int xr = WIDE ? mix_xr(nm) : NREG;
+    constexpr int xr = NREG;
     const float* Xp = sc.X + (size_t)li * xr * xr;
-    for_cols<WIDE, NW>(tid, n, [&](int c) {
+    for_col(lane, n, [&](int c) {
         if (obs_space) {
             const int oc = sm.lidx[c];
             const double sl = sm.lsq[c];
@@ -2710,8 +2693,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
         }
         for (int i = 0; i < n; ++i) sm.Y32[i * ld + c] = Xp[(size_t)i * xr + c];
     });
-    point_sync<NW>();
-    refine_rr<WIDE, NW>(sm.Ah, sm.Al, sm.Y32, sm.Wh, sm.Wl, sm.E32, sm.Ah, sm.dS, n, ld, tid);
+    __syncwarp();
+    refine_rr(sm.Ah, sm.Al, sm.Y32, sm.Wh, sm.Wl, sm.E32, sm.Ah, sm.dS, n, ld, lane);
     const float* E32 = sm.E32;
     const float* Soff = sm.Ah;  // S' off the diagonal; its diagonal is dS
     float* Y32 = sm.Y32;
@@ -2726,9 +2709,9 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
         const float af = (float)aa;
         const float rf = sqrtf(af);
         // d-hat in binary32, once (t2f is free until t2 is formed).
-        for (int l = tid; l < n; l += NTH) sm.t2f[l] = (float)sm.ldh[l];
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        for (int l = lane; l < n; l += 32) sm.t2f[l] = (float)sm.ldh[l];
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             const float ap = af + (float)sm.dS[c];  // a + s_ii
             const float u = sqrtf(ap);
             sm.vu[c] = u;
@@ -2739,8 +2722,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
             for (int l = 0; l < n; ++l) t += Y32[l * ld + c] * sm.t2f[l];
             sm.t1f[c] = t;
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             // t2 = h(S) t1 with h(S)_ii = h_i, h(S)_ij = -s_ij h_i h_j, and the
             // basis factor: minus E o (h_i + h_j)/2.
             const float hi = sm.vf[c];
@@ -2768,8 +2751,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
                 F32[i * ld + c] = v - E32[i * ld + c] * (0.5f * (gc - aj / rf));
             }
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             float t = 0.0f;
             for (int l = 0; l < n; ++l) t += Y32[c * ld + l] * sm.t2f[l];
             sm.vf[c] = t;  // v = (a I + A)^{-1} d-hat
@@ -2787,13 +2770,13 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
 #pragma unroll
             for (int a = 0; a < 9; ++a) sm.Z[a * nm + c] = sl * acc[a];
         });
-        point_sync<NW>();
-        if (tid < 9) {
+        __syncwarp();
+        if (lane < 9) {
             float s = 0.0f;
-            for (int i = 0; i < n; ++i) s += sm.Z[tid * nm + i] * sm.vf[i];
-            sm.zv[tid] = s;
+            for (int i = 0; i < n; ++i) s += sm.Z[lane * nm + i] * sm.vf[i];
+            sm.zv[lane] = s;
         }
-        for_cols<WIDE, NW>(tid, n, [&](int col) {
+        for_col(lane, n, [&](int col) {
             float acc[9];
 #pragma unroll
             for (int a = 0; a < 9; ++a) acc[a] = 0.0f;
@@ -2805,8 +2788,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
 #pragma unroll
             for (int a = 0; a < 9; ++a) sm.B[a * nm + col] = acc[a];  // Z Y
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int col) {
+        __syncwarp();
+        for_col(lane, n, [&](int col) {
             float acc[9];
 #pragma unroll
             for (int a = 0; a < 9; ++a) acc[a] = 0.0f;
@@ -2818,8 +2801,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
 #pragma unroll
             for (int a = 0; a < 9; ++a) sm.Z[a * nm + col] = acc[a];  // Z Y g(S)
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int col) {
+        __syncwarp();
+        for_col(lane, n, [&](int col) {
             float acc[9];
 #pragma unroll
             for (int a = 0; a < 9; ++a) acc[a] = 0.0f;
@@ -2832,9 +2815,9 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
 #pragma unroll
             for (int a = 0; a < 9; ++a) sm.B[a * nm + col] = sl * acc[a];  // sqrt(k-1) Z g(A) sqrt(rho)
         });
-        point_sync<NW>();
+        __syncwarp();
         const float sb = (float)sqrt(beta);
-        for (int m = tid; m < k; m += NTH) {
+        for (int m = lane; m < k; m += 32) {
             float acc[9];
 #pragma unroll
             for (int a = 0; a < 9; ++a) acc[a] = sm.xbar[a] + sm.zv[a] + sb * sm.dX[a * k + m];
@@ -2849,9 +2832,9 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
     } else {
         // Functions of S directly: 1/lambda for P-tilde, lambda^{-1/2} for W,
         // evaluated in binary32 (they enter binary32 products only).
-        for (int l = tid; l < n; l += NTH) sm.vf[l] = (float)sm.vb[l];  // b, once (vf is free until w-bar)
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        for (int l = lane; l < n; l += 32) sm.vf[l] = (float)sm.vb[l];  // b, once (vf is free until w-bar)
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             const float lam = (float)sm.dS[c];
             sm.vu[c] = sqrtf(lam);
             sm.vinv[c] = 1.0f / lam;
@@ -2859,8 +2842,8 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
             for (int l = 0; l < n; ++l) t += Y32[l * ld + c] * sm.vf[l];
             sm.t1f[c] = t;  // Y^T b
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             // t2 = f1(S) t1, f1(S)_ii = 1/l_i, f1(S)_ij = -s_ij / (l_i l_j), and
             // the basis factor: minus E o (f1_i + f1_j)/2.
             const float fc1 = (float)sm.vinv[c];
@@ -2885,32 +2868,32 @@ __global__ void __launch_bounds__(32 * NW) analyze_mixed_kernel(float* __restric
                 F32[i * ld + c] = v - E32[i * ld + c] * (0.5f * (1.0f / si + 1.0f / sj));
             }
         });
-        point_sync<NW>();
+        __syncwarp();
         float* YF = sm.Al;  // A's low half is no longer needed
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        for_col(lane, n, [&](int c) {
             float t = 0.0f;
             for (int l = 0; l < n; ++l) t += Y32[c * ld + l] * sm.t2f[l];
             sm.vf[c] = t;  // w-bar
         });
-        point_sync<NW>();
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        __syncwarp();
+        for_col(lane, n, [&](int c) {
             for (int i = 0; i < n; ++i) {
                 float s = 0.0f;
                 for (int l = 0; l < n; ++l) s += Y32[i * ld + l] * F32[l * ld + c];
                 YF[i * ld + c] = s;
             }
     });
-        point_sync<NW>();
+        __syncwarp();
         // T = sqrt(k-1) Y f2(S) Y^T + w-bar 1^T, over F32.
-        for_cols<WIDE, NW>(tid, n, [&](int c) {
+        for_col(lane, n, [&](int c) {
             for (int i = 0; i < n; ++i) {
                 float s = 0.0f;
                 for (int l = 0; l < n; ++l) s += YF[i * ld + l] * Y32[c * ld + l];
                 F32[i * ld + c] = sk * s + sm.vf[i];
             }
     });
-        point_sync<NW>();
-        for (int m = tid; m < k; m += NTH) {
+        __syncwarp();
+        for (int m = lane; m < k; m += 32) {
             for (int a = 0; a < 9; ++a) {
                 float s = 0.0f;
                 for (int j = 0; j < k; ++j) s += sm.dX[a * k + j] * F32[j * ld + m];
@@ -3031,7 +3014,9 @@ static cudaError_t launch_gram_mode(int nx, int ny, int k, const ObsParams& o, d
         if (k <= 64) return go(local_gram_fp64_kernel<64>);
         return go(local_gram_fp64_kernel<128>);
     } else if constexpr (MODE == PROD_DF32) {
-        if (k <= 64) return go(local_gram_df_kernel<64>);  // k > kOuterMaxK
+        if (k <= 16) return go(local_gram_df_kernel<16>);
+        if (k <= 32) return go(local_gram_df_kernel<32>);
+        if (k <= 64) return go(local_gram_df_kernel<64>);
         return go(local_gram_df_kernel<128>);
     } else {
         if (k <= 16) return go(local_gram_kernel<16>);
@@ -3106,12 +3091,13 @@ static cudaError_t launch_gram(int prod, int nx, int ny, int k, const ObsParams&
     return launch_gram_tc<false>(nx, ny, k, o, d_cut, aa, cell0, nc, sc, flags, s);
 }
 
-// Whether the double-binary32 Gram goes through the points' outer products:
-// up to kOuterMaxK members. Above, the rows themselves are multiplied
-// (local_gram_df_kernel): the other form's C differs from this one's at 1e-13,
-// which changes the binary32 matrix that kernel (A) starts from at 0.4% of
-// the grid points at k = 64, and the binary32 transform of such a point then
-// differs by up to three units in the last place (up to one for k <= 32).
+// Whether the double-binary32 Gram goes through the points' outer products
+// first: up to kOuterMaxK members. The two forms' C differ at ~1e-14, and
+// where that changes C rounded to binary32, which kernel (A) starts from, the
+// basis and with it the roundings of the whole transform change (seven units
+// in the last place of the state at worst). So local_gram_df_kernel then
+// recomputes the blocks with an entry that close to a rounding boundary. At
+// k = 64 most blocks have one, and the rows alone are quicker.
 static bool gram_by_outer(int npts, int kg, int prod) {
     return kg && kg <= kOuterMaxK && prod == PROD_DF32 && npts > 0;
 }
@@ -3145,8 +3131,10 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         const auto kernA = big ? mixed_jacobi_wide_kernel<64> : mixed_jacobi_wide_kernel<32>;
         const size_t shA = big ? WideShape<64>::bytes() : WideShape<32>::bytes();
         const int thA = big ? WideShape<64>::NT : WideShape<32>::NT;
-        const auto kernB = analyze_mixed_kernel<false, false, 1>;
-        if (!wide) {
+        const auto kernB = analyze_mixed_kernel;
+        // Kernel (B) from register tiles; up to 16 a tile leaves most of a warp idle.
+        const bool tiled = nm > 16;
+        if (!tiled) {
             e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
             if (e != cudaSuccess) return e;
         }
@@ -3196,7 +3184,8 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
                 ga.Clo = sc.Clo;
                 ga.b64 = sc.b64;
                 if ((e = launch_gram_outer(ga, (k - 1) / beta, aux->s2)) != cudaSuccess) return e;
-            } else if (kg && (e = launch_gram(prod, nx, ny, k, o, d_cut, (k - 1) / beta, (int)c0, nc, sc, flags,
+            }
+            if (kg && (e = launch_gram(prod, nx, ny, k, o, d_cut, (k - 1) / beta, (int)c0, nc, sc, flags,
                                        aux->s2)) != cudaSuccess)
                 return e;
             if (nm <= NREG && runA > 1)
@@ -3209,7 +3198,7 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
                 kernA<<<(unsigned)nc, thA, shA, aux->s2>>>(nx, ny, k, o, d_cut, beta, (int)c0, nm, sc, flags);
             if ((e = cudaEventRecord(aux->jac_done[b], aux->s2)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(s, aux->jac_done[b], 0)) != cudaSuccess) return e;
-            if (wide) {
+            if (tiled) {
                 const WideArgs wa{(float*)f, nx,      ny,        k,       o,      d_cut,  beta,   (int)c0, nm, sc.X,
                                   mix_xr(nm), sc.lsq, sc.lidx, sc.pcount, sc.C32, sc.Clo, sc.C64, sc.b32,  sc.b64, flags};
                 if ((e = launch_analyze_wide(wa, nc, s)) != cudaSuccess) return e;

@@ -1,4 +1,4 @@
-// Kernel (B) of the mixed-precision analysis for local problems of 33..128
+// Kernel (B) of the mixed-precision analysis for local problems of 17..128
 // (sm_103a): the refinement and transform of analyze_mixed_kernel
 // (letkf_kernels.cu; arXiv 2308.03972, Section 3.2) by a block per grid
 // point, with every n^3 product from register tiles.
@@ -32,7 +32,7 @@ struct WideB {
     static constexpr int T = NCG * NRG;
     static constexpr int LD = (KP + 31) / 32 * 32;
     static constexpr int MAT = KP * LD;
-    // 64: 55 KB, four blocks per SM; 96: two; above, one.
+    // 32: 16 KB, one warp, twelve per SM; 64: 55 KB, four blocks; 96: two; above, one.
     static size_t bytes(int k) {
         return sizeof(float) * (3 * (size_t)MAT + 10 * (size_t)KP + 9 * (size_t)k + 32) +
                KP * (3 * sizeof(double) + sizeof(int));
@@ -92,6 +92,10 @@ __device__ __forceinline__ void tile_mul_df(const float* __restrict__ Ah, const 
                                             const float* __restrict__ B, int n, int ti, int tj, f2x (&s)[4][4],
                                             f2x (&c)[4][4]) {
     using RS = WideB<KP>;
+    // One iteration is ~160 packed instructions; unrolled by four the three
+    // products overflow the instruction cache up to 64 (B at 256^2: 5.9 -> 3.6 ms
+    // at n = 32, 21.9 -> 18.9 at 64); above, one block per SM gains by it.
+#pragma unroll (KP <= 64 ? 1 : 4)
     for (int k = 0; k < n; ++k) {
         const int sw = (k >> 2) & 7;
         const int o0 = k * RS::LD + ((ti ^ sw) << 2), o1 = k * RS::LD + (((RS::NRG + ti) ^ sw) << 2);
@@ -118,6 +122,7 @@ __device__ __forceinline__ void sym_mul_df(const float* __restrict__ A, const fl
                                            const float* __restrict__ Bl, int n, int ri, int tj, f2x (&s)[4][4],
                                            f2x (&c)[4][4]) {
     using RS = WideB<KP>;
+#pragma unroll (KP <= 64 ? 1 : 4)
     for (int k = 0; k < n; ++k) {
         const int sw = (k >> 2) & 7;
         const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(A + k * RS::LD + (((2 * ri) ^ sw) << 2));
@@ -194,7 +199,7 @@ __device__ __forceinline__ void tile_store_t(float* M, int ti, int tj, const flo
 }
 
 template <int KP>
-__global__ void __launch_bounds__(WideB<KP>::T, KP <= 64 ? 4 : (KP <= 96 ? 2 : 1)) analyze_wide_kernel(WideArgs g) {
+__global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : (KP <= 96 ? 2 : 1))) analyze_wide_kernel(WideArgs g) {
     using RS = WideB<KP>;
     constexpr int LD = RS::LD, T = RS::T, NW = T / 32;  // full warps
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -572,6 +577,7 @@ cudaError_t launch_kp(const WideArgs& g, int ncell, cudaStream_t s) {
 }  // namespace
 
 cudaError_t launch_analyze_wide(const WideArgs& g, int ncell, cudaStream_t s) {
+    if (g.nm <= 32) return launch_kp<32>(g, ncell, s);
     if (g.nm <= 48) return launch_kp<48>(g, ncell, s);
     if (g.nm <= 64) return launch_kp<64>(g, ncell, s);
     if (g.nm <= 80) return launch_kp<80>(g, ncell, s);
