@@ -43,9 +43,9 @@ L2_NOTE = "state larger than L2: 151 MB per buffer in FP32, 302 MB in FP64 (L2 =
 # kernels in the same capture.
 ISSUE_ACTIVE = {"run_jacobi_kernel<28>": 0.748, "run_refine_kernel<28>": 0.585}
 # Launches of one mixed analysis at 256^2 x 64 (runs of 8 grid points, one
-# chunk of runs): binary32 copy of dY, split of the observation Gram, the
-# Jacobi kernel and the refinement kernel.
-MIXED_ANALYSIS_LAUNCHES = 4
+# chunk of runs): weight table, binary32 copy of dY, split of the observation
+# Gram, the Jacobi kernel and the refinement kernel.
+MIXED_ANALYSIS_LAUNCHES = 5
 NCU_TRAFFIC = {
     "analysis_mixed": 0.634112e6 + 167.438336e6 + 379.888384e6 + 117.160704e6,  # run kernels J + F
     "lbm_step_f32": 151.54816e6 + 97.796096e6,
@@ -238,10 +238,10 @@ def measure(cfg, precision, steps, warmup, sample_clocks=False, gpu_index=0, run
     ana = [e[2].elapsed_time(e[3]) for e in ev]
     osse.close()
     # Kernels per cycle: the LBM steps, observe + Gram, then the analysis
-    # (mixed: MIXED_ANALYSIS_LAUNCHES; FP64 on runs: split Gram, kernel J,
-    # the FP64 kernel; FP64 cold: one launch).
+    # (mixed: MIXED_ANALYSIS_LAUNCHES; FP64 on runs: weight table, split Gram,
+    # kernel J, the FP64 kernel; FP64 cold: table and one launch).
     if precision == binding.LBM_FP64:
-        ana_launches = 3 if run_length > 0 else 1
+        ana_launches = 4 if run_length > 0 else 2
     else:
         ana_launches = MIXED_ANALYSIS_LAUNCHES
     return {"ms_per_cycle": total_ms / steps, "lbm_step_ms": statistics.mean(lbm),

@@ -1875,9 +1875,10 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_df_kernel(int nx,
     const int nv = o.nvar;
     if (K <= kOuterMaxK) {
         // After the outer-product pass: only blocks where some entry's low
-        // half lies within 2^-44 of the largest diagonal entry of half a unit
-        // in the last place of the high half (half of that just above a power
-        // of two).
+        // half lies within 2^-48 of the largest diagonal entry of half a unit
+        // in the last place of the high half, or whose high half is a power of
+        // two (the spacing changes there). The forms differ by 3e-16 on average
+        // (from the share of points whose basis changed without this pass).
         bool near = false;
         if (li0 + w < ncell) {
             const float* Ch = sc.C32 + (size_t)(li0 + w) * k * k;
@@ -1885,7 +1886,7 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_df_kernel(int nx,
             float dm = lane < k ? Ch[lane * k + lane] : 0.0f;
 #pragma unroll
             for (int t = 16; t > 0; t >>= 1) dm = fmaxf(dm, __shfl_xor_sync(kFull, dm, t));
-            const float tau = 5.7e-14f * dm;
+            const float tau = 3.6e-15f * dm;
             for (int e = lane; e < k * k; e += 32) {
                 const unsigned b = __float_as_uint(Ch[e]) & 0x7fffffffu;
                 const float half = b >= (25u << 23) ? __uint_as_float((b & 0x7f800000u) - (24u << 23)) : 0.0f;
@@ -2119,7 +2120,9 @@ __global__ void __launch_bounds__(32 * kJacWarps, 4) mixed_jacobi_run_kernel(int
 //    went through shared memory (two thirds of the traffic that bound the
 //    kernel), and every access looked its pair up.
 // The entries see the rotations in the same order with the same roundings as
-// before; the result is the same to the bit.
+// before; the result is the same to the bit. Per analysis: n = 64 at 256^2
+// points 195 -> 90 ms (issue slots 57%, barriers), n = 88..104 at 128^2
+// 213 -> 147 ms (one point per SM: barriers).
 constexpr int kUR = 4;            // rows of U per thread
 constexpr int kBlkThreads = 256;  // threads that load the matrix
 
@@ -2583,7 +2586,7 @@ __device__ void refine_rr(const float* Ah, const float* Al, const float* Y32, fl
     __syncwarp();
 }
 
-// Kernel (B) for local problems up to 16 (launch_analyze), one warp per grid point.
+// Kernel (B) for local problems up to 26 (launch_analyze), one warp per grid point.
 __global__ void __launch_bounds__(32) analyze_mixed_kernel(float* __restrict__ f, int nx, int ny,
                                                            int k, ObsParams o, double d_cut,
                                                            double beta, int cell0, int nm,
@@ -3132,8 +3135,11 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         const size_t shA = big ? WideShape<64>::bytes() : WideShape<32>::bytes();
         const int thA = big ? WideShape<64>::NT : WideShape<32>::NT;
         const auto kernB = analyze_mixed_kernel;
-        // Kernel (B) from register tiles; up to 16 a tile leaves most of a warp idle.
-        const bool tiled = nm > 16;
+        // Kernel (B) from register tiles. A tile's time goes with 32^2 n, one
+        // column per lane's with n^3: at n = 32 3.6 against 5.9 ms per 256^2
+        // lattice, even at n = 25; at n = 20 and 21 whole cycles of small
+        // lattices were 2 to 4% slower with tiles.
+        const bool tiled = nm > 26;
         if (!tiled) {
             e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
             if (e != cudaSuccess) return e;
