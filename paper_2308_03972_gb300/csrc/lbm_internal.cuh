@@ -126,9 +126,8 @@ struct AnalyzeAux {
     cudaEvent_t start, jac_done[2], ref_done[2];
 };
 // Scratch the analysis needs (bytes; 0 for the FP64 path).
-// nl: capacity of a local list (ObsParams::plmax, or nobs); npts: observation
-// points.
-size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int npts, int nmax, int k, int prod);
+// nl: capacity of a local list (ObsParams::plmax, or nobs).
+size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int nmax, int k, int prod);
 // nmax: largest local problem size n = min(p, k) over the grid (sizes the
 // mixed kernel's shared memory; points above it are reported as too large).
 // prod: PROD_* arithmetic of the ensemble-space Gram (mixed precision only),
@@ -152,28 +151,6 @@ cudaError_t launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t 
 size_t weight_table_bytes(int nx, int ny);
 int weight_table_entries(int nx, int ny, double d_cut);
 cudaError_t launch_weight_table(const ObsParams& o, double d_cut, int entries, double* tab, cudaStream_t s);
-
-// ---- letkf_gram.cu --------------------------------------------------------
-// Double-binary32 Gram of the grid points cell0 .. of a chunk through the
-// observation points' outer products O, R (gram_outer_bytes bytes at an
-// 8-byte aligned base, filled by launch_outer): C = C32 + Clo [ncell][k][k],
-// b64 [ncell][k].
-struct GramArgs {
-    int nx, ny, k;
-    ObsParams o;
-    double d_cut;
-    int cell0 = 0, ncell = 0;
-    float2* O = nullptr;
-    double* R = nullptr;
-    float* C32 = nullptr;
-    float* Clo = nullptr;
-    double* b64 = nullptr;
-};
-constexpr int kOuterMaxK = 32;  // members
-size_t gram_outer_bytes(int npts, int k);
-void gram_outer_at(void* base, int npts, int k, GramArgs* g);
-cudaError_t launch_outer(const GramArgs& g, cudaStream_t s);
-cudaError_t launch_gram_outer(const GramArgs& g, double aa, cudaStream_t s);
 
 // ---- letkf_wide.cu --------------------------------------------------------
 // Refinement and update (kernel (B)) of the grid points cell0 .. of a chunk

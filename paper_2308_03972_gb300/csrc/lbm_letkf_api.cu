@@ -563,7 +563,7 @@ int analyze_prepare(lbm_ctx* c, double d_cut, double beta, AnalysisPlan* plan, b
         if (maxunion <= kRunMaxUnion) run_len = c->run_len;
     }
     const size_t scratch = run_len > 0 ? run_scratch_bytes(c->nx, c->ny, c->nvar * c->npts, run_len, maxunion, whole)
-                                       : analyze_scratch_bytes(c->nx, c->ny, is_fp32(c), plmax, c->npts, nmax, c->k, prod);
+                                       : analyze_scratch_bytes(c->nx, c->ny, is_fp32(c), plmax, nmax, c->k, prod);
     if (scratch > c->ana_scratch_bytes) {
         CK(c, cudaStreamSynchronize(c->stream), "synchronising");
         cudaFree(c->ana_scratch);

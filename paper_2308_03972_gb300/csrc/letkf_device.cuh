@@ -102,21 +102,6 @@ __device__ __forceinline__ void df_acc1(float& s, float& c, float a, float y) {
     c = __fadd_rn(c, __fadd_rn(t, e));
 }
 
-// A double-binary32 sum (s, c), plus (ah + al) when diag, renormalised into
-// binary32 high and low halves (Fast2Sum: the compensated sum's s dominates).
-__device__ __forceinline__ void df_pair_out(float s, float c, bool diag, float ah, float al, float& hi,
-                                            float& lo) {
-    if (diag) {
-        float t, e;
-        two_sum(s, ah, t, e);
-        c = __fadd_rn(c, __fadd_rn(e, al));
-        s = t;
-    }
-    const float h = __fadd_rn(s, c);
-    hi = h;
-    lo = __fsub_rn(c, __fsub_rn(h, s));
-}
-
 __device__ __forceinline__ double df_value(float s, float c) { return (double)s + (double)c; }
 
 // ---- Packed binary32 pairs (sm_100 family: add/sub/mul/fma .f32x2) --------

@@ -1830,6 +1830,21 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_fp64_kernel(int n
         if (lane + 32 * c < k) sc.b64[(size_t)li * k + lane + 32 * c] = bacc[c];
 }
 
+// A double-binary32 sum (s, c), plus (ah + al) when diag, renormalised into
+// binary32 high and low halves (Fast2Sum: the compensated sum's s dominates).
+__device__ __forceinline__ void df_pair_out(float s, float c, bool diag, float ah, float al, float& hi,
+                                            float& lo) {
+    if (diag) {
+        float t, e;
+        two_sum(s, ah, t, e);
+        c = __fadd_rn(c, __fadd_rn(e, al));
+        s = t;
+    }
+    const float h = __fadd_rn(s, c);
+    hi = h;
+    lo = __fsub_rn(c, __fsub_rn(h, s));
+}
+
 // Double-binary32 Gram (PROD_DF32, the default of a mixed-precision
 // context): the C and b of the FP64 Gram pass to FP64-class accuracy on the
 // binary32 units. The staged rows are split once into binary32 halves
@@ -1873,28 +1888,6 @@ __global__ void __launch_bounds__(32 * kGramPts, 1) local_gram_df_kernel(int nx,
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int li0 = blockIdx.x * kGramPts;
     const int nv = o.nvar;
-    if (K <= kOuterMaxK) {
-        // After the outer-product pass: only blocks where some entry's low
-        // half lies within 2^-48 of the largest diagonal entry of half a unit
-        // in the last place of the high half, or whose high half is a power of
-        // two (the spacing changes there). The forms differ by 3e-16 on average
-        // (from the share of points whose basis changed without this pass).
-        bool near = false;
-        if (li0 + w < ncell) {
-            const float* Ch = sc.C32 + (size_t)(li0 + w) * k * k;
-            const float* Cl = sc.Clo + (size_t)(li0 + w) * k * k;
-            float dm = lane < k ? Ch[lane * k + lane] : 0.0f;
-#pragma unroll
-            for (int t = 16; t > 0; t >>= 1) dm = fmaxf(dm, __shfl_xor_sync(kFull, dm, t));
-            const float tau = 3.6e-15f * dm;
-            for (int e = lane; e < k * k; e += 32) {
-                const unsigned b = __float_as_uint(Ch[e]) & 0x7fffffffu;
-                const float half = b >= (25u << 23) ? __uint_as_float((b & 0x7f800000u) - (24u << 23)) : 0.0f;
-                near |= fabsf(fabsf(Cl[e]) - half) <= tau || ((b & 0x7fffffu) == 0u && b != 0u);
-            }
-        }
-        if (!__syncthreads_or(near)) return;
-    }
     const int total = gram_merge(o, nx, ny, d_cut, cell0, li0, ncell, U, pcnt, wcount);
     const long long lim2 = support_lim2(d_cut);
     const float aah = (float)aa, aal = (float)(aa - (double)aah);  // a = aah + aal
@@ -3094,25 +3087,13 @@ static cudaError_t launch_gram(int prod, int nx, int ny, int k, const ObsParams&
     return launch_gram_tc<false>(nx, ny, k, o, d_cut, aa, cell0, nc, sc, flags, s);
 }
 
-// Whether the double-binary32 Gram goes through the points' outer products
-// first: up to kOuterMaxK members. The two forms' C differ at ~1e-14, and
-// where that changes C rounded to binary32, which kernel (A) starts from, the
-// basis and with it the roundings of the whole transform change (seven units
-// in the last place of the state at worst). So local_gram_df_kernel then
-// recomputes the blocks with an entry that close to a rounding boundary. At
-// k = 64 most blocks have one, and the rows alone are quicker.
-static bool gram_by_outer(int npts, int kg, int prod) {
-    return kg && kg <= kOuterMaxK && prod == PROD_DF32 && npts > 0;
-}
-
-size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int npts, int nmax, int k, int prod) {
+size_t analyze_scratch_bytes(int nx, int ny, int fp32, int nl, int nmax, int k, int prod) {
     if (!fp32) return 0;
     const int nm = mixed_nm(nmax);
     const int kg = gram_k(fp32, k, prod), gsz = gram_sz(prod);
     const long long cells = (long long)nx * ny;
     const long long chunk = mix_chunk(cells, nl, nm, kg, gsz);
-    return (chunk < cells ? 2 : 1) * mix_buf_bytes(chunk, nl, nm, kg, gsz) +  // double-buffered
-           (gram_by_outer(npts, kg, prod) ? gram_outer_bytes(npts, kg) : 0);
+    return (chunk < cells ? 2 : 1) * mix_buf_bytes(chunk, nl, nm, kg, gsz);  // double-buffered
 }
 
 cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsParams& o,
@@ -3169,12 +3150,6 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         // scratch is double-buffered, (A) of chunk c waits for (B) of c-2.
         if ((e = cudaEventRecord(aux->start, s)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(aux->s2, aux->start, 0)) != cudaSuccess) return e;
-        const bool outer = gram_by_outer(o.npts, kg, prod);
-        GramArgs ga{nx, ny, k, o, d_cut};
-        if (outer) {
-            gram_outer_at((unsigned char*)scratch + (chunk < cells ? 2 : 1) * buf_bytes, o.npts, k, &ga);
-            if ((e = launch_outer(ga, aux->s2)) != cudaSuccess) return e;
-        }
         int c = 0;
         for (long long c0 = 0; c0 < cells; c0 += chunk, ++c) {
             const int nc = (int)((cells - c0) < chunk ? (cells - c0) : chunk);
@@ -3183,14 +3158,6 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
             if (prod == PROD_DF32) sc = mix_scratch_df2(sc, chunk, kg);
             if (c >= 2 && (e = cudaStreamWaitEvent(aux->s2, aux->ref_done[b], 0)) != cudaSuccess)
                 return e;
-            if (outer) {
-                ga.cell0 = (int)c0;
-                ga.ncell = nc;
-                ga.C32 = sc.C32;
-                ga.Clo = sc.Clo;
-                ga.b64 = sc.b64;
-                if ((e = launch_gram_outer(ga, (k - 1) / beta, aux->s2)) != cudaSuccess) return e;
-            }
             if (kg && (e = launch_gram(prod, nx, ny, k, o, d_cut, (k - 1) / beta, (int)c0, nc, sc, flags,
                                        aux->s2)) != cudaSuccess)
                 return e;
