@@ -5,9 +5,12 @@
 //
 // A thread owns an 8 x 4 tile of a product (two groups of four rows). Each
 // entry's sum runs over the inner index in order with the roundings of the
-// one-column-per-lane form, so the results agree with it to the bit; per
-// multiply-add it needs 3 / 32 shared 16-byte loads where that form needed
-// two to four 4-byte ones and was bound by them. Three matrices are held in
+// one-column-per-lane form, and S' is corrected in FP64 as there, so the
+// results agree with it to the bit (but for entries of E and S whose sum of
+// two halves is a binary32 tie after rounding to binary64, which that form
+// rounds twice: about one in 2^29); per multiply-add it needs 3 / 32 shared
+// 16-byte loads where that form needed two to four 4-byte ones and was bound
+// by them. Three matrices are held in
 // shared memory (A and then A Y as binary32 halves, and the basis), reused as
 // the analysis proceeds; above 64 the older form kept A and A Y in global
 // scratch.
@@ -22,6 +25,7 @@
 
 #include "lbm_internal.cuh"
 #include "letkf_device.cuh"
+#include "vec.cuh"
 
 namespace lbmgpu {
 namespace {
@@ -213,9 +217,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
     float* vinv = vu + KP;
     float* t1 = vinv + KP;
     float* t2 = t1 + KP;
-    float* dh = t2 + KP;  // diagonal of S as binary32 halves
-    float* dl = dh + KP;
-    float* vb = dl + KP;  // and two more, for the nine rows of R0 below
+    float* vb = t2 + KP;  // and four more, for the nine rows of R0 below
     float* dX = vf + 10 * KP;  // [9][k]
     float* xbar = dX + 9 * g.k;
     float* zv = xbar + 10;
@@ -356,19 +358,15 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int i = 8 * ri + q;
-                    if (i == 4 * cj + j) {
-                        const double d = df_value(sv[q][j], vc[q][j]);
-                        const float h = (float)d;
-                        dS[i] = d;
-                        dh[i] = h;
-                        dl[i] = (float)(d - (double)h);
-                    }
+                    if (i == 4 * cj + j) dS[i] = df_value(sv[q][j], vc[q][j]);
                     sv[q][j] = __fadd_rn(sv[q][j], vc[q][j]);
                 }
         }
         __syncthreads();
-        // S' = S - E o (d_i + d_j)/2 off the diagonal, to both triangles, the
-        // correction in double-binary32.
+        // S' = S - E o (d_i + d_j)/2 off the diagonal, to both triangles, in
+        // FP64 with one rounding to binary32 (two operations per entry, the
+        // conversions on the integer units: 0.2 ms per 256^2 points at n = 32,
+        // 0.7 at 64).
         if (mine) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
@@ -377,13 +375,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
                     const int i = 8 * ri + q, c = 4 * cj + j;
                     if (i > c) continue;
                     const float e = ev[q][j];
-                    float th, tl;
-                    two_sum(dh[i], dh[c], th, tl);
-                    tl = __fadd_rn(tl, __fadd_rn(dl[i], dl[c]));
-                    const float e2 = 0.5f * e;
-                    const float pr = __fmul_rn(e2, th);
-                    const float pe = __fmaf_rn(e2, tl, __fmaf_rn(e2, th, -pr));
-                    const float s = __fsub_rn(__fsub_rn(sv[q][j], pr), pe);
+                    const float s = narrow(fma(-widen(0.5f * e), dS[i] + dS[c], widen(sv[q][j])));
                     M1[at<LD>(i, c)] = s;
                     M1[at<LD>(c, i)] = s;
                     M2[at<LD>(i, c)] = e;

@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 EXPECTED = analysis_words.load(os.path.join(os.path.dirname(os.path.abspath(__file__)), "golden", "analysis_words.txt"))
 
 
-@pytest.mark.parametrize("name", ["dense_16", "density_24", "scalars_28", "scalars_60"])
+@pytest.mark.parametrize("name", sorted(analysis_words.CASES))
 def test_posterior_words(gpu, name):
     got = analysis_words.rows(gpu, name)
     assert len(got) == len(EXPECTED[name])
