@@ -114,6 +114,9 @@ cudaError_t launch_store_force(void* dst, int fp32, const double* src, size_t n,
                                cudaStream_t s);
 
 // ---- letkf_kernels.cu -----------------------------------------------------
+// Largest ensemble that the observation operator takes (3 k + 12 doubles in
+// 48 KB of shared memory).
+constexpr int kObsMaxMembers = 2044;
 cudaError_t launch_observe(const void* f, int fp32, int nx, int ny, int k, int npts, int nvar,
                            const int* ix, const int* iy, const double* yo, double* dY,
                            double* d, cudaStream_t s);

@@ -39,11 +39,14 @@ struct WideB {
     static constexpr int LD = (KP + 31) / 32 * 32;
     static constexpr int MAT = KP * LD;
     // 32: 16 KB, one warp, twelve per SM; 64: 55 KB, four blocks; 96: two; above, one.
-    static size_t bytes(int k) {
-        return sizeof(float) * (3 * (size_t)MAT + 10 * (size_t)KP + 9 * (size_t)k + 32) +
+    // kdx: members whose perturbations are staged (k, or 0).
+    static constexpr size_t bytes(int kdx) {
+        return sizeof(float) * (3 * (size_t)MAT + 10 * (size_t)KP + 9 * (size_t)kdx + 32) +
                KP * (3 * sizeof(double) + sizeof(int));
     }
 };
+
+constexpr size_t kMaxShared = 227 * 1024;
 
 // Element group g (four columns) of row i: groups are permuted within
 // 128-byte lines by the row's group, so that walking a column block along
@@ -204,7 +207,12 @@ __device__ __forceinline__ void tile_store_t(float* M, int ti, int tj, const flo
     }
 }
 
-template <int KP>
+// STAGED: the perturbations dX [9][k] are held in shared memory. Otherwise
+// (ensembles that do not fit beside the matrices: from 751 members at KP = 128,
+// from 1,464 at 112; always in observation space) they are formed from the
+// state at each use; a thread's own values are the last it reads before it
+// writes them.
+template <int KP, bool STAGED>
 __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : (KP <= 96 ? 2 : 1))) analyze_wide_kernel(WideArgs g) {
     using RS = WideB<KP>;
     constexpr int LD = RS::LD, T = RS::T, NW = T / 32;  // full warps
@@ -219,9 +227,10 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
     float* t2 = t1 + KP;
     float* vb = t2 + KP;  // and four more, for the nine rows of R0 below
     float* dX = vf + 10 * KP;  // [9][k]
-    float* xbar = dX + 9 * g.k;
+    const int kdx = STAGED ? g.k : 0;
+    float* xbar = dX + 9 * kdx;
     float* zv = xbar + 10;
-    double* dS = reinterpret_cast<double*>(dX + 9 * g.k + 32 - (g.k & 1));
+    double* dS = reinterpret_cast<double*>(dX + 9 * kdx + 32 - (kdx & 1));
     double* lsq = dS + KP;
     double* ldh = lsq + KP;
     int* lidx = reinterpret_cast<int*>(ldh + KP);
@@ -239,13 +248,15 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
         float s = 0.0f;
         for (int m = lane; m < k; m += 32) {
             const float xv = fc[a * plane + m];
-            dX[a * k + m] = xv;
+            if (STAGED) dX[a * k + m] = xv;
             s += xv;
         }
         const float mean = warp_sum(s) / (float)k;
-        for (int m = lane; m < k; m += 32) dX[a * k + m] -= mean;
+        if (STAGED)
+            for (int m = lane; m < k; m += 32) dX[a * k + m] -= mean;
         if (lane == 0) xbar[a] = mean;
     }
+    auto dx = [&](int a, int m) { return STAGED ? dX[a * k + m] : __fsub_rn(fc[a * plane + m], xbar[a]); };
     const int p = g.pcount[li];
     if (p > cap) {
         if (tid == 0) atomicOr(g.flags, FLAG_TOOLARGE);
@@ -269,7 +280,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
     if (p == 0) {
         const float sb = (float)sqrt(g.beta);
         for (int a = 0; a < 9; ++a)
-            for (int m = tid; m < k; m += T) fc[a * plane + m] = xbar[a] + sb * dX[a * k + m];
+            for (int m = tid; m < k; m += T) fc[a * plane + m] = xbar[a] + sb * dx(a, m);
         return;
     }
     const double aa = (k - 1) / g.beta;
@@ -458,7 +469,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
         for (int l = 0; l < n; ++l) t += Yt[at<LD>(l, c)] * t2[l];
         vf[c] = t;
     }
-    if (!obs_space) {
+    if (STAGED && !obs_space) {  // n = k <= KP: staged
         const int n4 = (n + 3) & ~3;
         f2x acc[4][4];
         tile_zero(acc);
@@ -500,7 +511,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
         for (int m = 0; m < k; ++m) {
             const float dy = row[m];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) acc[a] += dX[(a0 + a) * k + m] * dy;
+            for (int a = 0; a < 3; ++a) acc[a] += dx(a0 + a, m) * dy;
         }
         const float sl = (float)lsq[c];
 #pragma unroll
@@ -547,7 +558,7 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
         const int m = e % k, a0 = e / k * 3;
         float acc[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) acc[a] = xbar[a0 + a] + zv[a0 + a] + sb * dX[(a0 + a) * k + m];
+        for (int a = 0; a < 3; ++a) acc[a] = xbar[a0 + a] + zv[a0 + a] + sb * dx(a0 + a, m);
         for (int i = 0; i < n; ++i) {
             const float dy = g.o.dY32[(size_t)lidx[i] * k + m];
 #pragma unroll
@@ -560,11 +571,16 @@ __global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : 
 
 template <int KP>
 cudaError_t launch_kp(const WideArgs& g, int ncell, cudaStream_t s) {
-    const size_t sh = WideB<KP>::bytes(g.k);
-    const cudaError_t e =
-        cudaFuncSetAttribute(analyze_wide_kernel<KP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    size_t sh = WideB<KP>::bytes(g.k);
+    auto kern = analyze_wide_kernel<KP, true>;
+    if constexpr (WideB<KP>::bytes(kObsMaxMembers) > kMaxShared)
+        if (sh > kMaxShared) {
+            sh = WideB<KP>::bytes(0);
+            kern = analyze_wide_kernel<KP, false>;
+        }
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     if (e != cudaSuccess) return e;
-    analyze_wide_kernel<KP><<<(unsigned)ncell, WideB<KP>::T, sh, s>>>(g);
+    kern<<<(unsigned)ncell, WideB<KP>::T, sh, s>>>(g);
     return cudaGetLastError();
 }
 
