@@ -298,7 +298,6 @@ struct AnaSmem {
     double* zv;    // [16]
     double* rc;    // [NM / 2]
     double* rs;    // [NM / 2]
-    float* Zf;     // [9][NM] binary32
     int* rp;       // [NM / 2]
     int* rq;       // [NM / 2]
     int* lidx;     // [nl]
@@ -306,7 +305,7 @@ struct AnaSmem {
     __host__ __device__ static size_t bytes(int k, int nl) {
         const size_t d = 2 * (size_t)NM * kLd + 9 * (size_t)k + 16 + 2 * (size_t)nl + 5 * NM +
                          18 * (size_t)NM + 16 + NM;
-        return d * sizeof(double) + 9 * NM * sizeof(float) + (size_t)(NM + nl) * sizeof(int);
+        return d * sizeof(double) + (size_t)(NM + nl) * sizeof(int);
     }
     __device__ void carve(unsigned char* raw, int k, int nl) {
         double* p = reinterpret_cast<double*>(raw);
@@ -342,8 +341,7 @@ struct AnaSmem {
         p += NM / 2;
         rs = p;
         p += NM / 2;
-        Zf = reinterpret_cast<float*>(p);
-        int* ip = reinterpret_cast<int*>(Zf + 9 * NM);
+        int* ip = reinterpret_cast<int*>(p);
         rp = ip;
         ip += NM / 2;
         rq = ip;
@@ -351,14 +349,6 @@ struct AnaSmem {
         lidx = ip;
     }
 };
-
-// 1 / d from the binary32 reciprocal and one Newton step (relative error
-// ~1e-13; here it scales entries that are ~1e-6 of the result).
-__device__ __forceinline__ double recip_step(double d) {
-    if (!(d > 1e-30 && d < 1e30)) return 1.0 / d;
-    const double r = widen(__fdividef(1.0f, narrow(d)));
-    return fma(r, fma(-d, r, 1.0), r);
-}
 
 // Largest off-diagonal entry (relative to a = (k-1)/beta) that the FP64
 // transform below takes as it is.
@@ -376,15 +366,17 @@ constexpr double kOffDiag = 1e-6;
 //        = -(1/r) (K0 + P)^{-1}, K0 = diag(1/alpha), alpha_i = 1/(u_i (u_i + r)),
 //   P = O + r (X1 + X2), X1_ij = O_ij / (u_i + u_j), X2_ij = -(X1^2)_ij / (u_i + u_j)
 // (X^2 = aI + S to second order), and (K0 + P)^{-1} = alpha - alpha P alpha +
-// alpha P alpha P alpha. What is neglected is third order: with |O_ij| <=
-// 1e-6 a (the eigensolve's stopping rule, or 3e-8 ||A||_F where that is
-// more) below 1e-14 of the transform, where the first-order functions that
-// stood here left 3e-13 at 3e-8 ||A||_F. So the eigensolve may stop an order
-// and a half earlier: from kernel J's basis it usually has nothing left to
-// rotate. Second-order terms (< 1e-9 of the result) run in binary32, scaled
-// by a so that they stay in its range. Once X1 is formed only the upper
-// triangle of A is used (P, FP64); each entry below the diagonal holds the
-// binary32 factor (X1 / r, then P / a) of the mirrored one.
+// alpha P alpha P alpha. What is neglected is third order in O / a, where the
+// eigensolve leaves |O_ij| <= max(1e-6 a, 3e-8 ||A||_F): at most 5e-16 of the
+// transform with every entry at 1e-6 a, the cube of 3e-8 ||A||_F / a for wider
+// spectra.
+// The first-order functions that stood here left the square of that (they
+// needed 3e-8 ||A||_F throughout), so the eigensolve may stop an order and a
+// half earlier: from kernel J's basis it usually has nothing left to rotate.
+// Error against FP64 singular values, max |f| = 1, for ||A||_F / a of 6e2, 2e4
+// and 4e5 (n = 32 and 48): first order 4e-14, 2e-11 and 4e-10, this form 8e-16,
+// 8e-15 and 4e-13. Everything is FP64. Once X1 is formed the upper triangle of A holds P and
+// the lower one X1.
 template <int NM>
 __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t plane, int k, int n,
                                 double aa, double beta, const ObsParams& o, int lane) {
@@ -392,7 +384,7 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
     double* A = sm.A;
     double* U = sm.U;
     auto up = [&](int i, int j) -> double& { return A[i < j ? i * ld + j : j * ld + i]; };
-    auto low = [&](int i, int j) -> float& { return *reinterpret_cast<float*>(A + (i > j ? i * ld + j : j * ld + i)); };
+    auto low = [&](int i, int j) -> double& { return A[i > j ? i * ld + j : j * ld + i]; };
     const double rr = sqrt(aa);
     const double ir = 1.0 / rr;
     for (int c = lane; c < n; c += 32) {
@@ -440,9 +432,9 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
             if (2 * d == n && c >= d) break;
             const int j = c + d < n ? c + d : c + d - n;
             const double off = A[j * ld + c];
-            const double x1 = off * recip_step(uc + sm.v3[j]);
+            const double x1 = off / (uc + sm.v3[j]);
             up(j, c) = fma(rr, x1, off);
-            low(j, c) = narrow(x1 * ir);
+            low(j, c) = x1;
         }
         double t = 0.0;
         for (int l = 0; l < n; ++l) t += U[c * ld + l] * sm.v2[l];
@@ -461,32 +453,29 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
         for (int a = 0; a < 9; ++a) sm.Z[a * NM + c] = sm.lsq[c] * acc[a];
     }
     __syncwarp();
-    // P += r X2 = -a q / (u_i / r + u_j / r), q = (X1 / r)^2 (its diagonal,
-    // too: P's diagonal is that term alone).
+    // P += r X2 = -r (X1^2) / (u_i + u_j) (its diagonal, too: P's diagonal is
+    // that term alone).
     for (int c = lane; c < n; c += 32) {
-        const float uc = narrow(sm.v3[c] * ir);
+        const double uc = sm.v3[c];
         for (int d = 0; 2 * d <= n; ++d) {
             if (2 * d == n && c >= d) break;
             const int j = c + d < n ? c + d : c + d - n;
-            float q0 = 0.0f, q1 = 0.0f;
+            double q0 = 0.0, q1 = 0.0;
             for (int l = 0; l < n; ++l) {
                 if (l == c || l == j) continue;
-                const float xa = low(l, c), xb = low(l, j);
+                const double xa = low(l, c), xb = low(l, j);
                 if (l & 1)
-                    q1 = fmaf(xa, xb, q1);
+                    q1 = fma(xa, xb, q1);
                 else
-                    q0 = fmaf(xa, xb, q0);
+                    q0 = fma(xa, xb, q0);
             }
-            const float x2 = __fdividef(q0 + q1, uc + narrow(sm.v3[j] * ir));
+            const double x2 = (q0 + q1) / (uc + sm.v3[j]);
             const double p1 = d == 0 ? 0.0 : up(j, c);
-            up(j, c) = fma(-aa, widen(x2), p1);
+            up(j, c) = fma(-rr, x2, p1);
         }
     }
     __syncwarp();
-    // P / a in binary32 below the diagonal; zv = Z v (= dX w-bar);
-    // B = Z U diag(alpha).
-    for (int c = lane; c < n; c += 32)
-        for (int i = 0; i < c; ++i) low(i, c) = narrow(A[i * ld + c] * (ir * ir));
+    // zv = Z v (= dX w-bar); B = Z U diag(alpha).
     if (lane < 9) {
         double s = 0.0;
         for (int i = 0; i < n; ++i) s += sm.Z[lane * NM + i] * sm.v1[i];
@@ -516,25 +505,21 @@ __device__ void fp64_obs_update(AnaSmem<NM>& sm, double* __restrict__ fc, size_t
             for (int a = 0; a < 9; ++a) acc[a] = fma(sm.B[a * NM + j], pj, acc[a]);
         }
 #pragma unroll
-        for (int a = 0; a < 9; ++a) {
-            const double z = sm.v5[c] * acc[a];
-            sm.Z[a * NM + c] = z;
-            sm.Zf[a * NM + c] = narrow(z * aa);
-        }
+        for (int a = 0; a < 9; ++a) sm.Z[a * NM + c] = sm.v5[c] * acc[a];
     }
     __syncwarp();
     for (int c = lane; c < n; c += 32) {
-        float acc[9];
+        double acc[9];
 #pragma unroll
-        for (int a = 0; a < 9; ++a) acc[a] = 0.0f;
+        for (int a = 0; a < 9; ++a) acc[a] = 0.0;
         for (int j = 0; j < n; ++j) {
-            const float pj = j == c ? narrow(A[c * ld + c] * (ir * ir)) : low(j, c);
+            const double pj = up(j, c);
 #pragma unroll
-            for (int a = 0; a < 9; ++a) acc[a] = fmaf(sm.Zf[a * NM + j], pj, acc[a]);
+            for (int a = 0; a < 9; ++a) acc[a] = fma(sm.Z[a * NM + j], pj, acc[a]);
         }
 #pragma unroll
         for (int a = 0; a < 9; ++a)
-            sm.B[a * NM + c] = fma(sm.v5[c], widen(acc[a]), sm.B[a * NM + c] - sm.Z[a * NM + c]);
+            sm.B[a * NM + c] = fma(sm.v5[c], acc[a], sm.B[a * NM + c] - sm.Z[a * NM + c]);
     }
     __syncwarp();
     // B <- -sqrt(k-1)/r B U^T diag(sqrt(rho)), ready to meet dY (through Z).

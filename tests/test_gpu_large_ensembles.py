@@ -6,31 +6,11 @@ import pytest
 
 import oracle
 from paper_2308_03972_gb300 import inputs
-from _helpers import U_RMS, W_REST, norm_rel, turbulent_state
+from _helpers import U_RMS, W_REST, norm_rel, svd_analysis, turbulent_state
 
 pytestmark = pytest.mark.gpu
 SIGMA = 0.1 * U_RMS
 BETA = 1.05
-
-
-def _exact(f, ix, iy, yu, yv, d_cut, x, y):
-    """The analysis of grid point (x, y) in FP64: C = a I + Yh^T Yh through the
-    singular values of Yh [p][k]; every observation is in range."""
-    ny, nx, k = f.shape[1:]
-    _, u, v = oracle.moments(f)
-    Y = np.stack([u[iy, ix], v[iy, ix]], 1).reshape(-1, k)
-    d = np.stack([yu, yv], 1).ravel() - Y.mean(1)
-    _, r = oracle.local_obs(nx, ny, x, y, ix, iy, SIGMA, SIGMA, d_cut)
-    lw = np.sqrt(r)
-    Yh = lw[:, None] * (Y - Y.mean(1, keepdims=True))
-    a = (k - 1) / BETA
-    U, s, Vt = np.linalg.svd(Yh, full_matrices=False)
-    wbar = Vt.T @ (s / (a + s * s) * (U.T @ (lw * d)))
-    X = f[:, y, x, :]
-    xm = X.mean(1, keepdims=True)
-    dX = X - xm
-    root = dX / np.sqrt(a) + (dX @ Vt.T) * (1.0 / np.sqrt(a + s * s) - 1.0 / np.sqrt(a)) @ Vt
-    return xm + (dX @ wbar)[:, None] + np.sqrt(k - 1.0) * root
 
 
 @pytest.mark.parametrize("k,nox,noy", [
@@ -57,5 +37,5 @@ def test_large_ensemble_matches_fp64(gpu, k, nox, noy):
     # 5e-8 of max |f| for binary32 sums up to 32 members, growing as their square root.
     tol = 5e-8 * np.sqrt(max(k, 32) / 32.0)
     for x, y in ((0, 0), (nx - 1, 0), (2, ny - 1), (nx // 2, ny // 2)):
-        ref = _exact(f, ix, iy, yu, yv, d_cut, x, y)
+        ref = svd_analysis(oracle, f, ix, iy, yu, yv, SIGMA, d_cut, BETA, x, y)
         assert norm_rel(got[:, y, x, :], ref) <= tol
