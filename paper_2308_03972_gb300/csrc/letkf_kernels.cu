@@ -729,7 +729,8 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
     const size_t plane = (size_t)nx * ny * k;
     double* fc = f + cell * k;
 
-    const double ik = 1.0 / k;
+    // Means: the nine divisions (FP64 pipe) in one instruction, lane a the a-th.
+    double mean = 0.0;
     for (int a = 0; a < 9; ++a) {
         double s = 0.0;
         for (int m = lane; m < k; m += 32) {
@@ -737,9 +738,14 @@ __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, in
             sm.dX[a * k + m] = xv;
             s += xv;
         }
-        const double mean = warp_sum(s) * ik;
-        for (int m = lane; m < k; m += 32) sm.dX[a * k + m] -= mean;
-        if (lane == 0) sm.xbar[a] = mean;
+        s = warp_sum(s);
+        if (lane == a) mean = s;
+    }
+    mean /= k;
+    if (lane < 9) sm.xbar[lane] = mean;
+    for (int a = 0; a < 9; ++a) {
+        const double ma = __shfl_sync(kFull, mean, a);
+        for (int m = lane; m < k; m += 32) sm.dX[a * k + m] -= ma;
     }
     const int* info = rinfo + (size_t)rl * info_stride;
     const int nu = info[0];
