@@ -142,7 +142,8 @@ int lbm_velocity_rmse(lbm_ctx *ctx, lbm_ctx *truth, double *rmse, int ptr_kind);
  * them all). FP64 in both precisions. With LBM_PTR_HOST the call
  * synchronises; the scratch it needs is allocated and released on the
  * context stream. LBM_EINVAL if nshells < 1 or the lattice is too large for
- * the diagnostic (nx or ny beyond about 1700). */
+ * the diagnostic (nx > 1614, or 56 ny + 8 s > 232448 with s = nshells, at
+ * most the number of shells above). */
 int lbm_energy_spectrum(lbm_ctx *ctx, double *E, int nshells, int ptr_kind);
 
 /* Observation step (Section 3, y = H x; Section 3.2, ybar and dY): record

@@ -173,16 +173,14 @@ __global__ void __launch_bounds__(kFftThreads) spectrum_rows_kernel(const T* __r
 }
 
 // Pass 2. Grid (nx, groups of G members). Shared: two buffers [ny][G]
-// complex, twiddles [ny], energies [ny], shell of each ky [ny]. Output
-// P [groups][nx][nsh].
+// complex, twiddles [ny]; the energies and the shell of each ky [ny] take the
+// buffer that the transform leaves free. Output P [groups][nx][nsh].
 __global__ void __launch_bounds__(kFftThreads) spectrum_cols_kernel(const double2* __restrict__ F1, int nx, int ny,
                                                                     int k, int G,
                                                                     const __grid_constant__ FftPlan plan, int nsh,
                                                                     double* __restrict__ P) {
     extern __shared__ __align__(16) double2 shz[];
     double2 *za = shz, *zb = za + (size_t)ny * G, *tw = zb + (size_t)ny * G;
-    double* e = reinterpret_cast<double*>(tw + ny);
-    int* shell = reinterpret_cast<int*>(e + ny);
     const int x = blockIdx.x;
     const int m0 = blockIdx.y * G;
     fft_twiddles(tw, ny);
@@ -191,6 +189,8 @@ __global__ void __launch_bounds__(kFftThreads) spectrum_cols_kernel(const double
         za[t] = m < k ? F1[((size_t)y * nx + x) * k + m] : make_double2(0.0, 0.0);
     }
     const double2* z = fft_block(za, zb, tw, plan, G);
+    double* e = reinterpret_cast<double*>(z == za ? zb : za);
+    int* shell = reinterpret_cast<int*>(e + ny);
     const int kx = 2 * x > nx ? x - nx : x;
     const double inv_n = 1.0 / ((double)nx * (double)ny);
     for (int y = threadIdx.x; y < ny; y += kFftThreads) {
@@ -271,35 +271,31 @@ __global__ void __launch_bounds__(kRmseThreads) rmse_final_kernel(const double* 
 
 constexpr size_t kMaxShared = 227 * 1024;
 
-static size_t rows_shared(int nx, int G) { return (2 * (size_t)G + 1) * nx * sizeof(double2); }
-static size_t cols_shared(int ny, int G) {
-    return (2 * (size_t)G + 1) * ny * sizeof(double2) + (size_t)ny * (sizeof(double) + sizeof(int));
-}
+static size_t fft_shared(int n, int G) { return (2 * (size_t)G + 1) * n * sizeof(double2); }
 
 // Members per block: eight (32- or 64-byte runs of f, 128-byte runs of F1)
 // while two blocks fit an SM, fewer on long rows and columns.
-template <typename F>
-static int spectrum_group(int n, F&& bytes) {
+static int spectrum_group(int n) {
     int G = 8;
-    while (G > 1 && bytes(n, G) > kMaxShared / 2) G /= 2;
+    while (G > 1 && fft_shared(n, G) > kMaxShared / 2) G /= 2;
     return G;
 }
 
 size_t spectrum_work_bytes(int nx, int ny, int k, int nshells) {
-    const int G = spectrum_group(ny, cols_shared);
+    const int G = spectrum_group(ny);
     return (size_t)k * ny * nx * sizeof(double2) + (size_t)((k + G - 1) / G) * nx * nshells * sizeof(double);
 }
 
 cudaError_t launch_energy_spectrum(const void* f, int fp32, int nx, int ny, int k, double* E,
                                    int nshells, void* work, int* flags, cudaStream_t s) {
     // The lattice sizes the diagnostic takes: rows of up to 1,614 cells, and
-    // columns and shells within 227 KB at 56 bytes a cell and 8 a shell.
+    // columns and shells within 227 KB at 56 bytes a cell and 8 a shell. One
+    // member per block needs 48 bytes a cell, so all of them fit.
     const size_t lim1 = (size_t)nx * 144, lim2 = 56 * (size_t)ny + 8 * (size_t)nshells;
     if (lim1 > kMaxShared || lim2 > kMaxShared) return cudaErrorInvalidValue;
-    const int G1 = spectrum_group(nx, rows_shared), G2 = spectrum_group(ny, cols_shared);
-    const size_t sh1 = rows_shared(nx, G1), sh2 = cols_shared(ny, G2);
+    const int G1 = spectrum_group(nx), G2 = spectrum_group(ny);
+    const size_t sh1 = fft_shared(nx, G1), sh2 = fft_shared(ny, G2);
     const int n1 = (k + G1 - 1) / G1, n2 = (k + G2 - 1) / G2;
-    if (sh1 > kMaxShared || sh2 > kMaxShared) return cudaErrorInvalidValue;
     double2* F1 = reinterpret_cast<double2*>(work);
     double* P = reinterpret_cast<double*>(F1 + (size_t)k * ny * nx);
     const FftPlan px = fft_plan(nx), py = fft_plan(ny);
