@@ -258,6 +258,11 @@ int observe_impl(lbm_ctx* c, int npts, const int* ix, const int* iy, const doubl
             return fail(c, LBM_EINVAL, "observation %d is not finite", j);
     }
     const int nobs = nvar * npts;
+    // The analysis' weight table, here because an FP64 context's first analysis
+    // allocates nothing and may be captured. Sized by the lattice, so a captured
+    // analysis keeps its address.
+    if (!c->wtab)
+        CK(c, cudaMalloc(&c->wtab, weight_table_bytes(c->nx, c->ny)), "allocating weight table");
     if (!c->obs_copied)
         CK(c, cudaEventCreateWithFlags(&c->obs_copied, cudaEventDisableTiming), "creating event");
     if (npts > c->pts_cap || nobs > c->nobs_cap) {
@@ -572,9 +577,6 @@ int analyze_prepare(lbm_ctx* c, double d_cut, double beta, AnalysisPlan* plan, b
         CK(c, cudaMalloc(&c->ana_scratch, scratch), "allocating analysis scratch");
         c->ana_scratch_bytes = scratch;
     }
-    // Sized by the lattice, so a captured analysis keeps its address.
-    if (!c->wtab)
-        CK(c, cudaMalloc(&c->wtab, weight_table_bytes(c->nx, c->ny)), "allocating weight table");
     if ((is_fp32(c) || run_len > 0) && !c->aux_ready) {
         CK(c, cudaStreamCreateWithFlags(&c->aux.s2, cudaStreamNonBlocking), "creating stream");
         CK(c, cudaEventCreateWithFlags(&c->aux.start, cudaEventDisableTiming), "creating event");
