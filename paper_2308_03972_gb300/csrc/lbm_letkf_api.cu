@@ -344,15 +344,22 @@ cudaError_t scratch_pool(lbm_ctx* c) {
 }
 
 // Device buffers of one call, allocated and released in stream order on the
-// context stream.
+// context stream. While the stream is captured they are the graph's own
+// (allocation nodes), and no pool is made.
 struct StreamScratch {
     lbm_ctx* c;
     std::vector<void*> bufs;
     explicit StreamScratch(lbm_ctx* ctx) : c(ctx) {}
     cudaError_t get(void** p, size_t bytes) {
         *p = nullptr;
-        cudaError_t e = scratch_pool(c);
-        if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, c->pool, c->stream);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaStreamIsCapturing(c->stream, &cap);
+        if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) {
+            e = cudaMallocAsync(p, bytes ? bytes : 16, c->stream);
+        } else {
+            if (e == cudaSuccess) e = scratch_pool(c);
+            if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, c->pool, c->stream);
+        }
         if (e == cudaSuccess) bufs.push_back(*p);
         return e;
     }
