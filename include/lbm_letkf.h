@@ -140,8 +140,8 @@ int lbm_velocity_rmse(lbm_ctx *ctx, lbm_ctx *truth, double *rmse, int ptr_kind);
  * over members. E[nshells] receives shells s = 0 .. nshells-1; wavenumbers in
  * higher shells are dropped (floor(hypot(nx/2, ny/2) + 1/2) + 1 shells hold
  * them all). FP64 in both precisions. With LBM_PTR_HOST the call
- * synchronises; the scratch it needs is allocated and released on the
- * context stream. LBM_EINVAL if nshells < 1 or the lattice is too large for
+ * synchronises; the scratch it needs is stream-ordered and kept for later
+ * calls (see lbm_destroy). LBM_EINVAL if nshells < 1 or the lattice is too large for
  * the diagnostic (nx > 1614, or 56 ny + 8 s > 232448 with s = nshells, at
  * most the number of shells above). */
 int lbm_energy_spectrum(lbm_ctx *ctx, double *E, int nshells, int ptr_kind);
@@ -256,8 +256,8 @@ int lbm_misfit(lbm_ctx *ctx, const lbm_window *win, double *J);
  * J stays a host array [members]. Any output may be NULL. In mixed
  * precision the forecast and the adjoint run in binary32 (C_s derivative
  * summed in FP64); in FP64 mode everything is FP64. Scratch of about
- * (nsteps / checkpoint_every + checkpoint_every + 3) states is allocated
- * and released on the context stream. Synchronises. */
+ * (nsteps / checkpoint_every + checkpoint_every + 3) states is stream-ordered
+ * and kept for later calls (see lbm_destroy). Synchronises. */
 int lbm_misfit_gradient(lbm_ctx *ctx, const lbm_window *win, const double *w, double *J,
                         double *grad_f0, double *grad_cs, double *dcs, int ptr_kind);
 
@@ -314,7 +314,12 @@ int lbm_sync(lbm_ctx *ctx);
  * failed lbm_init or letkf_analyze_noalloc on this thread). Never NULL. */
 const char *lbm_last_error(const lbm_ctx *ctx);
 
-/* Free the context and its device buffers (synchronises its stream). */
+/* Free the context and its device buffers (synchronises its stream). The
+ * scratch of lbm_misfit, lbm_misfit_gradient, lbm_energy_spectrum,
+ * lbm_velocity_rmse and letkf_probe_transform stays with the context until
+ * then: at most 16 GiB over all contexts of the process, and none where an
+ * allocation of this library would fail without it. Other allocators of the
+ * process do not see it as free. */
 void lbm_destroy(lbm_ctx *ctx);
 
 /* Limits of letkf_analyze_noalloc. */
