@@ -317,9 +317,9 @@ const char *lbm_last_error(const lbm_ctx *ctx);
 /* Free the context and its device buffers (synchronises its stream). The
  * scratch of lbm_misfit, lbm_misfit_gradient, lbm_energy_spectrum,
  * lbm_velocity_rmse and letkf_probe_transform stays with the context until
- * then: at most 16 GiB over all contexts of the process, and none where an
- * allocation of this library would fail without it. Other allocators of the
- * process do not see it as free. */
+ * then, at most 16 GiB over all contexts of the process. cudaMemGetInfo counts
+ * it as used; the driver takes it back where a cudaMalloc of the process would
+ * otherwise fail. */
 void lbm_destroy(lbm_ctx *ctx);
 
 /* Limits of letkf_analyze_noalloc. */

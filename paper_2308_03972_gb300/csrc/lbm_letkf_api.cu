@@ -104,8 +104,8 @@ bool ptr_kind_ok(int kind) { return kind == LBM_PTR_HOST || kind == LBM_PTR_DEVI
 // synchronisation, and mapping the 5 GB of a 256^2 x 64 gradient anew took 8 of
 // its 56 ms. All pools of the process together keep at most kPoolKeep (checked
 // when a call releases its buffers: the other contexts' unused memory goes
-// first), a pool is given back at lbm_destroy, and an allocation that fails is
-// tried again after all of them have given back what is unused.
+// first), and a pool is given back at lbm_destroy. The driver takes unused pool
+// memory back by itself where a cudaMalloc would otherwise fail.
 constexpr unsigned long long kPoolKeep = 16ull << 30;
 
 struct PoolRegistry {
@@ -135,22 +135,6 @@ void bound_pools(cudaMemPool_t own) {
         }
         total = std::min(total + v, kPoolKeep);
     }
-}
-
-void release_pools() {
-    PoolRegistry& r = pool_registry();
-    std::lock_guard<std::mutex> lock(r.m);
-    for (cudaMemPool_t p : r.pools) cudaMemPoolTrimTo(p, 0);
-}
-
-// cudaMalloc, once more without the pools' unused memory if it fails.
-template <typename T>
-cudaError_t device_alloc(T** p, size_t bytes) {
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e != cudaErrorMemoryAllocation) return e;
-    cudaGetLastError();
-    release_pools();
-    return cudaMalloc(p, bytes);
 }
 
 cudaError_t scratch_pool(lbm_ctx* c) {
@@ -192,7 +176,7 @@ void destroy_pool(lbm_ctx* c) {
 
 int ensure_stage(lbm_ctx* c) {
     if (c->stage) return LBM_OK;
-    CK(c, device_alloc(&c->stage, state_elems(c) * sizeof(double)), "allocating staging buffer");
+    CK(c, cudaMalloc(&c->stage, state_elems(c) * sizeof(double)), "allocating staging buffer");
     return LBM_OK;
 }
 
@@ -354,20 +338,20 @@ int observe_impl(lbm_ctx* c, int npts, const int* ix, const int* iy, const doubl
     // allocates nothing and may be captured. Sized by the lattice, so a captured
     // analysis keeps its address.
     if (!c->wtab)
-        CK(c, device_alloc(&c->wtab, weight_table_bytes(c->nx, c->ny)), "allocating weight table");
+        CK(c, cudaMalloc(&c->wtab, weight_table_bytes(c->nx, c->ny)), "allocating weight table");
     if (!c->obs_copied)
         CK(c, cudaEventCreateWithFlags(&c->obs_copied, cudaEventDisableTiming), "creating event");
     if (npts > c->pts_cap || nobs > c->nobs_cap) {
         CK(c, cudaStreamSynchronize(c->stream), "synchronising");
         free_obs(c);
         const size_t no = (size_t)nobs;
-        CK(c, device_alloc(&c->ix, 2 * npts * sizeof(int)), "allocating obs");
+        CK(c, cudaMalloc(&c->ix, 2 * npts * sizeof(int)), "allocating obs");
         c->iy = c->ix + npts;
-        CK(c, device_alloc(&c->yo, no * sizeof(double)), "allocating obs");
-        CK(c, device_alloc(&c->dY, no * c->k * sizeof(double)), "allocating obs");
-        CK(c, device_alloc(&c->d, no * sizeof(double)), "allocating obs");
-        CK(c, device_alloc(&c->G, no * no * sizeof(double)), "allocating obs");
-        if (is_fp32(c)) CK(c, device_alloc(&c->dY32, no * c->k * sizeof(float)), "allocating obs");
+        CK(c, cudaMalloc(&c->yo, no * sizeof(double)), "allocating obs");
+        CK(c, cudaMalloc(&c->dY, no * c->k * sizeof(double)), "allocating obs");
+        CK(c, cudaMalloc(&c->d, no * sizeof(double)), "allocating obs");
+        CK(c, cudaMalloc(&c->G, no * no * sizeof(double)), "allocating obs");
+        if (is_fp32(c)) CK(c, cudaMalloc(&c->dY32, no * c->k * sizeof(float)), "allocating obs");
         CK(c, cudaMallocHost(&c->h_yo, no * sizeof(double)), "allocating pinned staging");
         CK(c, cudaMallocHost(&c->h_ixy, 2 * npts * sizeof(int)), "allocating pinned staging");
         c->pts_cap = npts;
@@ -428,11 +412,6 @@ struct StreamScratch {
         } else {
             if (e == cudaSuccess) e = scratch_pool(c);
             if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, c->pool, c->stream);
-            if (e == cudaErrorMemoryAllocation && c->pool) {
-                cudaGetLastError();
-                release_pools();
-                e = cudaMallocFromPoolAsync(p, bytes ? bytes : 16, c->pool, c->stream);
-            }
             pooled = true;
         }
         if (e == cudaSuccess) bufs.push_back(*p);
@@ -657,7 +636,7 @@ int analyze_prepare(lbm_ctx* c, double d_cut, double beta, AnalysisPlan* plan, b
         cudaFree(c->ana_scratch);
         c->ana_scratch = nullptr;
         c->ana_scratch_bytes = 0;
-        CK(c, device_alloc(&c->ana_scratch, scratch), "allocating analysis scratch");
+        CK(c, cudaMalloc(&c->ana_scratch, scratch), "allocating analysis scratch");
         c->ana_scratch_bytes = scratch;
     }
     if ((is_fp32(c) || run_len > 0) && !c->aux_ready) {
@@ -773,12 +752,12 @@ int lbm_init(const lbm_config* cfg, const double* f0, const double* force, int p
     };
     const size_t bytes = state_elems(c) * elem_size(c);
     for (int b = 0; b < 2; ++b) {
-        cudaError_t e = device_alloc(&c->f[b], bytes);
+        cudaError_t e = cudaMalloc(&c->f[b], bytes);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "allocating state"));
     }
-    cudaError_t e = device_alloc(&c->force, (size_t)2 * c->nx * c->ny * elem_size(c));
+    cudaError_t e = cudaMalloc(&c->force, (size_t)2 * c->nx * c->ny * elem_size(c));
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "allocating force"));
-    e = device_alloc(&c->flags, sizeof(int));
+    e = cudaMalloc(&c->flags, sizeof(int));
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "allocating flags"));
     e = cudaMemsetAsync(c->flags, 0, sizeof(int), c->stream);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "clearing flags"));
@@ -787,7 +766,7 @@ int lbm_init(const lbm_config* cfg, const double* f0, const double* force, int p
     const size_t nf = (size_t)2 * c->nx * c->ny;
     if (force) {
         double* tmp = nullptr;
-        e = device_alloc(&tmp, nf * sizeof(double));
+        e = cudaMalloc(&tmp, nf * sizeof(double));
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "allocating force staging"));
         st = copy_in(c, tmp, force, nf, ptr_kind);
         if (st == LBM_OK) {
@@ -994,7 +973,7 @@ int letkf_set_run_length(lbm_ctx* c, int run_len) {
 int letkf_sweep_stats(lbm_ctx* c, int enable, int* hist) {
     if (!c) return fail(nullptr, LBM_EINVAL, "ctx is NULL");
     if (!c->sweep_hist) {
-        CK(c, device_alloc(&c->sweep_hist, 32 * sizeof(int)), "allocating sweep histogram");
+        CK(c, cudaMalloc(&c->sweep_hist, 32 * sizeof(int)), "allocating sweep histogram");
         CK(c, cudaMemsetAsync(c->sweep_hist, 0, 32 * sizeof(int), c->stream), "clearing sweep histogram");
     }
     if (hist) {
@@ -1102,7 +1081,7 @@ int lbm_nudge(lbm_ctx* c, int nobs_x, int nobs_y, const double* rho_o, const dou
         cudaFree(c->nudge_obs);
         c->nudge_obs = nullptr;
         c->nudge_cap = 0;
-        CK(c, device_alloc(&c->nudge_obs, 3 * no * sizeof(double)), "allocating nudging observations");
+        CK(c, cudaMalloc(&c->nudge_obs, 3 * no * sizeof(double)), "allocating nudging observations");
         c->nudge_cap = 3 * no;
     }
     // Copies from pageable memory are staged before the call returns.
@@ -1354,9 +1333,9 @@ int lbm_batch_create(lbm_ctx* const* ctxs, int n, lbm_batch** out) {
         lbm_batch_destroy(b);
         return code;
     };
-    cudaError_t e = device_alloc(&b->ex_dev, kMaxMultiExp * sizeof(MultiExp));
-    if (e == cudaSuccess) e = device_alloc(&b->bar, 4 * sizeof(unsigned));
-    if (e == cudaSuccess) e = device_alloc(&b->status, sizeof(int));
+    cudaError_t e = cudaMalloc(&b->ex_dev, kMaxMultiExp * sizeof(MultiExp));
+    if (e == cudaSuccess) e = cudaMalloc(&b->bar, 4 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMalloc(&b->status, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(b->status, 0, sizeof(int), b->stream);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming);
     if (e != cudaSuccess)
