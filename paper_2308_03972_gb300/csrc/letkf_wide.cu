@@ -38,8 +38,8 @@ struct WideB {
     static constexpr int T = NCG * NRG;
     static constexpr int LD = (KP + 31) / 32 * 32;
     static constexpr int MAT = KP * LD;
-    // 32: 16 KB, one warp, twelve per SM; 64: 55 KB, four blocks; 96: two; above, one.
-    // kdx: members whose perturbations are staged (k, or 0).
+    // 32: 16 KB, one warp, twelve per SM; 64: 55 KB, four blocks; 80: 101 KB, two;
+    // above, one. kdx: members whose perturbations are staged (k, or 0).
     static constexpr size_t bytes(int kdx) {
         return sizeof(float) * (3 * (size_t)MAT + 10 * (size_t)KP + 9 * (size_t)kdx + 32) +
                KP * (3 * sizeof(double) + sizeof(int));
@@ -213,7 +213,7 @@ __device__ __forceinline__ void tile_store_t(float* M, int ti, int tj, const flo
 // state at each use; a thread's own values are the last it reads before it
 // writes them.
 template <int KP, bool STAGED>
-__global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : (KP <= 96 ? 2 : 1))) analyze_wide_kernel(WideArgs g) {
+__global__ void __launch_bounds__(WideB<KP>::T, KP <= 32 ? 12 : (KP <= 64 ? 4 : (KP <= 80 ? 2 : 1))) analyze_wide_kernel(WideArgs g) {
     using RS = WideB<KP>;
     constexpr int LD = RS::LD, T = RS::T, NW = T / 32;  // full warps
     extern __shared__ __align__(16) unsigned char smem_raw[];
