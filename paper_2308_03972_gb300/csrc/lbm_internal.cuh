@@ -157,7 +157,7 @@ cudaError_t launch_weight_table(const ObsParams& o, double d_cut, int entries, d
 
 // ---- letkf_wide.cu --------------------------------------------------------
 // Refinement and update (kernel (B)) of the grid points cell0 .. of a chunk
-// with local problems up to nm, 26 < nm <= 128, from kernel (A)'s basis X
+// with local problems up to nm <= 128 (27 and up by launch_analyze's rule), from kernel (A)'s basis X
 // [.][xr][xr], local lists lsq, lidx and counts pcount, and the Gram pass's C
 // (C32 with or without Clo, or C64) and b (b32 or b64).
 struct WideArgs {

@@ -2570,7 +2570,7 @@ __device__ void refine_rr(const float* Ah, const float* Al, const float* Y32, fl
     __syncwarp();
 }
 
-// Kernel (B) for local problems up to 26 (launch_analyze), one warp per grid point.
+// Kernel (B) for local problems up to 32 (launch_analyze draws the line), one warp per grid point.
 __global__ void __launch_bounds__(32) analyze_mixed_kernel(float* __restrict__ f, int nx, int ny,
                                                            int k, ObsParams o, double d_cut,
                                                            double beta, int cell0, int nm,
@@ -3108,10 +3108,16 @@ cudaError_t launch_analyze(void* f, int fp32, int nx, int ny, int k, const ObsPa
         const int thA = big ? WideShape<64>::NT : WideShape<32>::NT;
         const auto kernB = analyze_mixed_kernel;
         // Kernel (B) from register tiles. A tile's time goes with 32^2 n, one
-        // column per lane's with n^3: at n = 32 3.6 against 5.9 ms per 256^2
-        // lattice, even at n = 25; at n = 20 and 21 whole cycles of small
-        // lattices were 2 to 4% slower with tiles.
-        const bool tiled = nm > 26;
+        // column per lane's with n^3. Whole analyses, one column against tiles:
+        // with ensemble-space points (n = k) 64^2 x 27 1.65 -> 1.59 ms,
+        // 256^2 x 32 23.9 -> 21.5; even at n = 25, and cycles of small lattices
+        // 2 to 4% slower at n = 20 and 21. In observation space the nine rows of
+        // Z, which both forms take column by column, grow with k: 28 scalars
+        // 0.94 -> 0.97 (k = 40) and 0.96 -> 1.04 ms (64); 30 scalars 1.28 -> 1.19
+        // and 1.33 -> 1.26, but 1.39 -> 1.50 at k = 128; 32 scalars 1.58 -> 1.39
+        // (64), 5.66 -> 6.85 (128, four times the points).
+        const bool ens = nmax >= k;  // some grid point in ensemble space
+        const bool tiled = nm > NREG || (ens ? nm > 26 : nm > 28 && k <= 64);
         if (!tiled) {
             e = cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shB);
             if (e != cudaSuccess) return e;

@@ -1,5 +1,5 @@
-// Kernel (B) of the mixed-precision analysis for local problems of 27..128
-// (sm_103a): the refinement and transform of analyze_mixed_kernel
+// Kernel (B) of the mixed-precision analysis for local problems of 33..128,
+// and of some of 27..32 (launch_analyze draws the line; sm_103a): the refinement and transform of analyze_mixed_kernel
 // (letkf_kernels.cu; arXiv 2308.03972, Section 3.2) by a block per grid
 // point, with every n^3 product from register tiles.
 //

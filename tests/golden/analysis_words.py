@@ -23,7 +23,8 @@ CASES = {
     "dense_64": (128, 64, 64, (16, 8), 24.0, 8, "DF32", False),
     "fp64_products_40": (64, 48, 40, (16, 12), 9.0, 8, "FP64", False),
     "members_128": (48, 32, 128, (12, 8), 40.0, 8, "DF32", False),
-    "scalars_28": (96, 96, 64, (12, 12), 8.5, 0, "DF32", False),
+    "scalars_32": (96, 96, 64, (12, 12), 8.5, 0, "DF32", False),
+    "scalars_32_of_128": (96, 64, 128, (12, 8), 8.5, 0, "DF32", False),
     "scalars_60": (96, 96, 96, (12, 12), 12.0, 8, "DF32", False),
     "scalars_100": (96, 96, 128, (12, 12), 16.0, 8, "DF32", False),
 }
