@@ -50,7 +50,7 @@ NCU_TRAFFIC = {
     "analysis_mixed": 0.634112e6 + 167.438336e6 + 379.888384e6 + 117.160704e6,  # run kernels J + F
     "lbm_step_f32": 151.54816e6 + 97.796096e6,
     # FP64 run path: kernel J (as in the mixed path) + run_fp64_kernel.
-    "analysis_fp64": 0.634112e6 + 167.438336e6 + 517.581568e6 + 251.356928e6,
+    "analysis_fp64": 0.634112e6 + 167.438336e6 + 532.26e6 + 253.72e6,
 }
 
 
@@ -392,10 +392,11 @@ def measure_adjoint(cfg, reps=3, nsteps=200, ckpt=20):
     ms = statistics.median(times)
     fms = statistics.median(ftimes)
     upd = nx * ny * k
-    # Algorithmic HBM bytes: forward 200 steps and recomputation of 180 (read
+    # Algorithmic HBM bytes: forward 200 steps and recomputation of 171 (every
+    # state between checkpoints but the last segment's, which is kept; read
     # + write 9 binary32 values), 200 adjoint steps (read f_t and lambda,
     # write lambda), the checkpoint copies, and the FP64 gradient write.
-    nrec = nsteps - nsteps // ckpt
+    nrec = ((nsteps + ckpt - 1) // ckpt - 1) * (ckpt - 1)
     byts = (nsteps + nrec) * 72 * upd + nsteps * 108 * upd + (nsteps // ckpt) * 72 * upd + 9 * 12 * upd
     return {"workload": "256x256 x 64 initial states, %d-step window, (u,v) misfit at 16x16 points every "
                         "10 steps, checkpoints every %d steps, binary32 forecast and adjoint" % (nsteps, ckpt),

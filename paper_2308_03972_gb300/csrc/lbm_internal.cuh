@@ -148,7 +148,7 @@ cudaError_t launch_to_f32(const double* src, float* dst, size_t n, cudaStream_t 
 // ObsParams::wtab: one entry per squared distance replaces the FP64 square
 // roots, divisions and polynomials of every (grid point, observation) pair
 // (FP64 issues at 1/64 of the binary32 rate; 256^2 x 16 with 32^2 points:
-// kernel (A) 5.6 -> 1.9 ms, the Gram 4.2 -> 1.8). weight_table_bytes: capacity
+// kernel (A) 5.6 -> 1.9 ms, the Gram 10.4 -> 6.5). weight_table_bytes: capacity
 // for a lattice (up to 8 MB); entries: used for d_cut, 0 where the capacity
 // does not hold them (the kernels then evaluate the weights themselves).
 size_t weight_table_bytes(int nx, int ny);

@@ -288,7 +288,7 @@ cudaError_t launch_step_v(const T* fin, T* fout, const T* force, const LbmParams
 // Moments from the stored state: rho = sum f, u = sum f c / rho, in FP64.
 // Bound by the FP64 pipe (two operations per SM cycle), so the nine
 // conversions run on the integer units and the sums share their differences:
-// 436 -> 291 us at 256^2 x 64 in binary32.
+// 436 -> 356 us at 256^2 x 64 in binary32.
 template <typename T, bool SHIFT>
 __global__ void moments_kernel(const T* __restrict__ f, int nx, int ny, int k,
                                double* __restrict__ rho, double* __restrict__ u,
@@ -309,8 +309,7 @@ __global__ void moments_kernel(const T* __restrict__ f, int nx, int ny, int k,
 // Ensemble-mean velocity of an FP64 state: one warp per cell, lanes over
 // members, moments and sum in FP64. The binary32 shifted state g = f - w has
 // its own kernel below, whose moments match that state's storage error
-// (~1e-9 absolute in u). One division per member: 479 -> 336 us at
-// 256^2 x 64.
+// (~1e-9 absolute in u). 479 -> 400 us at 256^2 x 64.
 __global__ void mean_velocity_kernel(const double* __restrict__ f, int nx, int ny, int k,
                                      double* __restrict__ um, double* __restrict__ vm,
                                      int* __restrict__ flags) {

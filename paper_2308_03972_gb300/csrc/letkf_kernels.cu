@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(32) analyze_fp64_kernel(double* __restrict__ f
 // The matrix functions are FP64's; the binary32 basis is only where the FP64
 // work starts. Bound by the FP64 pipe (two operations per SM cycle): two
 // rotating sweeps of the Jacobi were 200,000 of the kernel's 310,000
-// operations per grid point at n = 28, k = 64; 31.3 -> 18.0 ms per 256^2 x 64
+// operations per grid point at n = 28, k = 64; 31.3 -> 21.5 ms per 256^2 x 64
 // analysis without them.
 template <int NS>
 __global__ void __launch_bounds__(32) run_fp64_kernel(double* __restrict__ f, int nx, int ny, int k, ObsParams o,
@@ -2105,8 +2105,8 @@ __global__ void __launch_bounds__(32 * kJacWarps, 4) mixed_jacobi_run_kernel(int
 //    kernel), and every access looked its pair up.
 // The entries see the rotations in the same order with the same roundings as
 // before; the result is the same to the bit. Per analysis: n = 64 at 256^2
-// points 195 -> 90 ms (issue slots 57%, barriers), n = 88..104 at 128^2
-// 213 -> 147 ms (one point per SM: barriers).
+// points 195 -> 92 ms (issue slots 69%, barriers), n = 88..104 at 128^2
+// 213 -> 142 ms (one point per SM: barriers).
 constexpr int kUR = 4;            // rows of U per thread
 constexpr int kBlkThreads = 256;  // threads that load the matrix
 

@@ -18,8 +18,8 @@
 // Double-binary32 products bound the kernel: A Y (eleven operations per
 // multiply-add), and E = Y^T Y - I and S = Y^T (A Y), of which only the tiles
 // that reach the upper triangle are formed. Per analysis, one column per lane
-// against tiles: n = 64 at 256^2 points 59 -> 18.9 ms, n = 88..104 at 128^2
-// 54 -> 25.8 ms.
+// against tiles: n = 64 at 256^2 points 59 -> 19.6 ms, n = 88..104 at 128^2
+// 54 -> 26.1 ms.
 #include <cmath>
 #include <cstdint>
 
