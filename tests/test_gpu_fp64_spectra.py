@@ -6,7 +6,8 @@ import pytest
 
 import oracle
 from paper_2308_03972_gb300 import inputs
-from _helpers import TOL_FP64, U_RMS, norm_rel, svd_analysis, turbulent_state
+from _helpers import TOL_FP64, U_RMS, norm_rel, turbulent_state
+from _svd import svd_analysis
 
 pytestmark = pytest.mark.gpu
 

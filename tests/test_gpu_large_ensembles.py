@@ -6,7 +6,8 @@ import pytest
 
 import oracle
 from paper_2308_03972_gb300 import inputs
-from _helpers import U_RMS, W_REST, norm_rel, svd_analysis, turbulent_state
+from _helpers import U_RMS, W_REST, norm_rel, turbulent_state
+from _svd import svd_analysis
 
 pytestmark = pytest.mark.gpu
 SIGMA = 0.1 * U_RMS
