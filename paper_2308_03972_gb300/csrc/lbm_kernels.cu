@@ -417,53 +417,47 @@ __global__ void mean_velocity_f32_kernel(const float* __restrict__ f, int nx, in
     }
 }
 
-// f^eq(rho, u, v) of every member: f^eq_a - w_a = w_a (A + rho (4.5 (c.u)^2 +
-// 3 c.u)), A = rho - 1 - 1.5 rho u.u, in FP64. Opposite directions share their
-// even part; on a diagonal 4.5 (ux +- uy)^2 = 4.5 u.u +- 9 ux uy. Bound by
-// the FP64 pipe: about 30 operations per member-cell (and 9 additions of w in
-// FP64 storage), the conversions to binary32 on the integer units:
-// 517 -> 295 us at 256^2 x 64 in FP64.
-template <typename T, bool SHIFT>
+// f^eq(rho, u, v) of every member: f^eq_a - w_a = w_a q_a, q_a = (rho - 1) +
+// rho (4.5 (c.u)^2 + 3 c.u - 1.5 u.u), in FP64. The operations and their
+// roundings are fixed (a dense analysis makes a visible difference of a last
+// digit here): u.u = fma(ux, ux, uy uy), 4.5 (c.u)^2 as (4.5 c.u) c.u, each sum
+// an FMA. Opposite directions share that square. Bound by the FP64 pipe: about
+// 38 operations per member-cell (47 with RHO), 60 when every direction formed
+// its own, the conversions to binary32 on the integer units. 256^2 x 64, rho = 1
+// and given: 525 -> 305 and 384 us in FP64, 597 -> 320 and 397 us in binary32
+// (with rho tested per direction at run time 500).
+template <typename T, bool SHIFT, bool RHO>
 __global__ void equilibrium_kernel(T* __restrict__ f, size_t n, const double* __restrict__ rho,
                                    const double* __restrict__ u, const double* __restrict__ v) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double ux = u ? u[i] : 0.0, uy = v ? v[i] : 0.0;
-    double xx = ux * ux, yy = uy * uy, xy = ux * uy, lx = ux, ly = uy, r1 = 0.0;
-    if (rho) {
-        const double r = rho[i];
-        r1 = r - 1.0;
-        xx *= r;
-        yy *= r;
-        xy *= r;
-        lx *= r;
-        ly *= r;
-    }
-    const double uu = xx + yy;
-    const double A = fma(-1.5, uu, r1);
-    double d[9];
-    d[0] = (4.0 / 9.0) * A;
-    const double a1 = (1.0 / 9.0) * A;
-    const double ex = fma(0.5, xx, a1), ey = fma(0.5, yy, a1);
-    d[1] = fma(1.0 / 3.0, lx, ex);
-    d[2] = fma(-1.0 / 3.0, lx, ex);
-    d[3] = fma(1.0 / 3.0, ly, ey);
-    d[4] = fma(-1.0 / 3.0, ly, ey);
-    const double dg = (1.0 / 36.0) * fma(4.5, uu, A);
-    const double e5 = fma(0.25, xy, dg), e7 = fma(-0.25, xy, dg);
-    const double lp = lx + ly, lm = lx - ly;
-    d[5] = fma(1.0 / 12.0, lp, e5);
-    d[6] = fma(-1.0 / 12.0, lp, e5);
-    d[7] = fma(1.0 / 12.0, lm, e7);
-    d[8] = fma(-1.0 / 12.0, lm, e7);
+    const double r = RHO ? rho[i] : 1.0, r1 = r - 1.0;
+    const double uu = __fma_rn(ux, ux, __dmul_rn(uy, uy));
+    double x[9];  // 4.5 (c.u)^2 + 3 c.u
+    auto pair = [&](int a, double cu) {
+        const double sq = __dmul_rn(__dmul_rn(4.5, cu), cu);
+        x[a] = __fma_rn(3.0, cu, sq);
+        x[a + 1] = __fma_rn(-3.0, cu, sq);
+    };
+    x[0] = 0.0;
+    pair(1, ux);
+    pair(3, uy);
+    pair(5, ux + uy);
+    pair(7, ux - uy);
 #pragma unroll
-    for (int a = 0; a < 9; ++a) narrow_to(f[a * n + i], SHIFT ? d[a] : d2q9_w(a) + d[a]);
+    for (int a = 0; a < 9; ++a) {
+        double q = __fma_rn(-1.5, uu, x[a]);
+        if (RHO) q = __fma_rn(r, q, r1);
+        const double w = d2q9_w(a);
+        narrow_to(f[a * n + i], SHIFT ? __dmul_rn(w, q) : __fma_rn(w, q, w));
+    }
 }
 
 // FP64 f [9][ny][nx][k] <-> g = f - w in binary32 (plane = ny nx k; grid y = 9).
 // One FP64 addition per value is left on the FP64 pipe; the conversions run on
 // the integer units. With the equilibrium above, setting a
-// 256^2 x 64 binary32 ensemble and reading it back went from 744 to 393 us.
+// 256^2 x 64 binary32 ensemble and reading it back went from 744 to 466 us.
 __global__ void store_f_kernel(float* __restrict__ dst, const double* __restrict__ src, size_t plane) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= plane) return;
@@ -579,11 +573,11 @@ cudaError_t launch_set_equilibrium(void* f, int fp32, int nx, int ny, int k, con
                                    const double* u, const double* v, cudaStream_t s) {
     const size_t n = (size_t)nx * ny * k;
     if (n == 0) return cudaSuccess;
+    const auto go = [&](auto kern, auto* ff) { kern<<<blocks_for(n, 256), 256, 0, s>>>(ff, n, rho, u, v); };
     if (fp32)
-        equilibrium_kernel<float, true><<<blocks_for(n, 256), 256, 0, s>>>((float*)f, n, rho, u, v);
+        go(rho ? equilibrium_kernel<float, true, true> : equilibrium_kernel<float, true, false>, (float*)f);
     else
-        equilibrium_kernel<double, false><<<blocks_for(n, 256), 256, 0, s>>>((double*)f, n, rho, u,
-                                                                            v);
+        go(rho ? equilibrium_kernel<double, false, true> : equilibrium_kernel<double, false, false>, (double*)f);
     return cudaGetLastError();
 }
 

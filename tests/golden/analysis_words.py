@@ -1,7 +1,7 @@
-"""Words of mixed-precision analyses: a checksum of every lattice row's stored
-binary32 posterior, for inputs that are the same to the bit on any machine
-(uniform random numbers and sums of them, no libm). A kernel that sums in
-another order, or in other formats, changes some of them.
+"""Words of mixed-precision analyses and of the equilibrium: a checksum of every
+lattice row's result (stored binary32 posteriors), for inputs that are the same
+to the bit on any machine (uniform random numbers and sums of them, no libm). A
+kernel that sums in another order, or in other formats, changes some of them.
 
 ``python analysis_words.py FILE`` writes them for the package on ``sys.path``.
 """
@@ -57,7 +57,27 @@ def posterior(binding, name):
     return np.ascontiguousarray((out - w).astype(np.float32).transpose(1, 2, 0, 3))
 
 
+EQUILIBRIA = ("equilibrium_fp64", "equilibrium_fp64_rho", "equilibrium_mixed", "equilibrium_mixed_rho")
+
+
+def equilibrium(binding, name):
+    """f after set_equilibrium, [ny][nx][9][k]; its first row at rest."""
+    nx, ny, k = 250, 41, 24
+    rng = np.random.Generator(np.random.PCG64(7))
+    u, v = (rng.random((2, ny, nx, k)) - 0.5) * 0.2
+    u[0] = v[0] = 0.0
+    rho = 1.0 + (rng.random((ny, nx, k)) - 0.5) * 0.1 if name.endswith("_rho") else None
+    prec = binding.LBM_FP64 if "fp64" in name else binding.LBM_MIXED
+    with binding.Ensemble(nx, ny, k, 0.55, 0.2, 0.0, prec) as e:
+        e.set_equilibrium(rho, u, v)
+        out = e.get_f()
+        e.sync()
+    return np.ascontiguousarray(out.transpose(1, 2, 0, 3))
+
+
 def rows(binding, name):
+    if name in EQUILIBRIA:
+        return ["%08x" % zlib.crc32(r.tobytes()) for r in equilibrium(binding, name)]
     return ["%08x" % zlib.crc32(r.tobytes()) for r in posterior(binding, name)]
 
 
@@ -70,5 +90,5 @@ if __name__ == "__main__":
     from paper_2308_03972_gb300 import binding
 
     with open(sys.argv[1], "w") as fh:
-        for name in CASES:
+        for name in (*CASES, *EQUILIBRIA):
             fh.write(" ".join([name] + rows(binding, name)) + "\n")
